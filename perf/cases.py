@@ -257,7 +257,7 @@ def _prepare_hybrid(case, seed):
     converted by the first classification."""
     g = _gen(seed)
     nx, ny, nz = case["nx"], case["ny"], case["nz"]
-    inp = inputs.ramp_slab(nx=nx, ny=1, nz=1, a0=4.0, ppc=case["ppc"], slab_lambda=min(2.0, nx / 64.0),
+    inp = inputs.ramp_slab(nx=nx, ny=1, nz=1, a0=2.0, ppc=case["ppc"], slab_lambda=min(2.0, nx / 64.0),
                            vacuum_lambda=min(1.0, nx / 128.0))
     gr, bc = inp["grid"], inp["grid"]["bc"]
     laser = dict(inp["laser"], y_c=0.5 * (ny - 1), z_c=0.5 * (nz - 1))
@@ -269,9 +269,9 @@ def _prepare_hybrid(case, seed):
     n = (prof[None, None, :] * (1.0 + 0.02 * (_rand(g, nz, ny, nx) - 0.5))).cpu().numpy()
     for fl in inp["fluids"]:
         sim.load_fluid(fl["q"], fl["m"], n, n_floor=fl["n_floor"])
-    sim.set_fields(*_packet(g, nx, ny, nz, gr["dx"], 4.0, 0.3 * nx * gr["dx"], 0.08 * nx * gr["dx"],
+    sim.set_fields(*_packet(g, nx, ny, nz, gr["dx"], 2.0, 0.3 * nx * gr["dx"], 0.08 * nx * gr["dx"],
                             min(4.0 * math.pi, 0.2 * ny * gr["dx"]), bc))
-    model = Classifier(dropout=0.2, mc_passes=case["passes"], seed=11, std=[1.5] * 6, stream=sim.desc.stream)
+    model = Classifier(dropout=0.2, mc_passes=case["passes"], seed=11, std=[1.0] * 6, stream=sim.desc.stream)
     _set(model, _classifier_weights(11, out_bias=-4.0))
     sim.set_regime(dilate=2, ppc=case["ppc"], to_species=[0, 1], policy="union", reach=case["steps"] + 1)
     sim.classify(model)
