@@ -81,7 +81,10 @@ static void enqueue_step(hyb_ctx *c) {
     cudaMemsetAsync(c->mig_counts, 0, sizeof(int) * HYB_MAX_SPECIES, st);
     if (set.n > 0) {
         pm.begin(HYB_PH_PUSH);
-        launch_push_deposit(g, c->E, c->B, c->sp_dev, set.n, c->qed, c->jscratch, c->jvalid, c->status, c->step_dev,
+        bool events = false;
+        for (int i = 0; i < set.n; ++i)
+            events = events || set.s[i].zmax > 0 || set.s[i].qed || (set.s[i].kind == HYB_KIND_PHOTON && set.s[i].pair_e >= 0);
+        launch_push_deposit(g, c->E, c->B, c->sp_dev, set.n, events, c->qed, c->jscratch, c->jvalid, c->status, c->step_dev,
                             st);
         pm.end(HYB_PH_PUSH);
         pm.begin(HYB_PH_JREDUCE);
@@ -140,7 +143,12 @@ hyb_status alloc_slots(hyb_ctx *c, SpDev &s, int cap, bool has_zq, bool has_tau)
     if (ctx_alloc(c, (void **)&s.id, sizeof(uint64_t) * slots) || ctx_alloc(c, (void **)&s.holes, sizeof(int) * slots))
         return HYB_ENOMEM;
     // a particle moves less than one cell per step, so only the shell of a tile can leave it
-    const long long mig = std::min<long long>((long long)slots, std::max<long long>(65536, (long long)slots / 2));
+    long long mig = std::min<long long>((long long)slots, std::max<long long>(65536, (long long)slots / 2));
+    // room for the slots the push's warps leave unused in their last chunks: 8 warps a tile, of up to 4 CTAs a
+    // tile on grids small enough to be split.  A caller's arena was sized without it: no chunks there.
+    s.mig_chunks = c->arena.base ? 0 : 1;
+    if (s.mig_chunks)
+        mig += MIG_CHUNK * 8LL * std::max<long long>(c->g.ntiles, std::min<long long>(4LL * c->g.ntiles, 512));
     s.mig_cap = (int)std::min<long long>(mig, 0x7fffffffLL);
     float **ml[7] = {&s.mx, &s.my, &s.mz, &s.mux, &s.muy, &s.muz, &s.mw};
     for (auto f : ml)

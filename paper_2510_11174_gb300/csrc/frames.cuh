@@ -35,13 +35,66 @@ __device__ __forceinline__ int fix_exponent(double bound) {
     return k > 126 ? 126 : (k < -126 ? -126 : k);
 }
 
-// fixed-point image of a value already multiplied by 2^k
-__device__ __forceinline__ unsigned long long fix_of(float scaled) {
-    return (unsigned long long)__float2ll_rn(scaled);
+// Fixed-point image of a value already multiplied by 2^k (|value| < 2^62), the
+// nearest integer, as (low, high) words: the high digit by rounding the value
+// times 2^-32, the low one from the exact remainder.  (A remainder of exactly
+// 2^31, where the high digit ties, saturates one unit short.)  The conversion
+// instruction between FP32 and 64-bit integers runs on the FP64 pipe, which is
+// slow on this chip: it was 47 % busy in the push of 15.7 M thermal particles.
+__device__ __forceinline__ void fix_of(float scaled, unsigned &lo, unsigned &hi) {
+    const int h = __float2int_rn(scaled * 0x1p-32f);
+    const int l = __float2int_rn(fmaf(__int2float_rn(h), -0x1p32f, scaled));
+    lo = (unsigned)l;
+    hi = (unsigned)(h + (l >> 31));
 }
 
+// the FP32 nearest to a 64-bit sum (ties to even) times inv_scale (a power of
+// two).  Integer normalisation instead of the conversion instruction, as above.
 __device__ __forceinline__ float fix_to_float(unsigned long long s, float inv_scale) {
-    return __ll2float_rn((long long)s) * inv_scale;
+    const bool neg = (long long)s < 0;
+    const unsigned long long m = neg ? 0ULL - s : s;
+    if (m == 0ULL) return 0.0f;
+    const int z = __clzll((long long)m);
+    const unsigned long long n = m << z;           // leading bit at 63
+    const unsigned top = (unsigned)(n >> 32);
+    // 24 bits in the upper part of `top`, the guard bit and whether anything lies below it
+    unsigned q = top >> 8;
+    const unsigned rest = (top << 24) | ((unsigned)n != 0u ? 1u : 0u);
+    q += (rest > 0x80000000u || (rest == 0x80000000u && (q & 1u))) ? 1u : 0u;
+    // q 2^(40 - z): q <= 2^24 converts exactly; the exponent is in range for FP32
+    const float v = (float)(int)q * pow2f(40 - z);
+    return (neg ? -v : v) * inv_scale;
+}
+
+// A shared-memory frame of n nodes holds the n low words of its sums, then the
+// n high words.  A sum takes a value with two 32-bit atomics: the low word's
+// returns what it held, so the carry joins the high word's.  Shared memory adds
+// 32-bit integers natively, while a 64-bit atomicAdd there is a
+// compare-and-swap loop (15.7 M thermal particles with 12 to 54 contributions
+// each: 271 M -> 159 M shared-memory wavefronts).  Separate word planes keep
+// the accesses on all 32 banks.  The K low additions go out before the first
+// high one, so the K round trips overlap.  SKIP leaves out the values that are
+// 0 (most of a crossing particle's stencil).
+template <int K, bool SKIP = true>
+__device__ __forceinline__ void fix_add(unsigned *__restrict__ lo, int n, const int idx[K], const float scaled[K]) {
+    unsigned h[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        unsigned l;
+        fix_of(scaled[k], l, h[k]);
+        if (!SKIP || scaled[k] != 0.0f) {
+            const unsigned old = atomicAdd(lo + idx[k], l);
+            h[k] += old + l < l ? 1u : 0u;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+        if (!SKIP || h[k] != 0u) atomicAdd(lo + n + idx[k], h[k]);
+}
+
+// sum l of a frame of n nodes
+__device__ __forceinline__ unsigned long long fix_read(const unsigned *lo, int n, int l) {
+    return ((unsigned long long)lo[n + l] << 32) | lo[l];
 }
 
 // largest |v| over the block as the bits of a non-negative float (which order

@@ -130,6 +130,7 @@ struct SpDev {
     int *mdest;
     int *mig_count;
     int mig_cap;
+    int mig_chunks;        // the push's warps take MIG_CHUNK slots at a time (the buffer has room for what they waste)
     // field ionization (zmax = 0: none)
     int zmax;
     int ion_into;          // species index of the electrons
@@ -153,6 +154,11 @@ struct SpDev {
     // bit sp_index is set when a tile of this species passed half of its capacity
     int *fill_flags;
 };
+
+// Slots of the migration buffer that a warp of the push takes at a time.  One
+// atomic on a species' counter per 32 migrants instead of one per warp and
+// particle pass: they all hit one address and their latency is exposed.
+static constexpr int MIG_CHUNK = 32;
 
 // tallies per tile: energies (FP64) and event counts
 enum { TALLY_IONIZE = 0, TALLY_EMIT = 1, TALLY_PAIR = 2, NTALLY = 3 };
@@ -334,9 +340,9 @@ void launch_laser_source(const GridDev &g, const hyb_grid_desc &d, const float *
 void launch_step_inc(long long *step_dev, cudaStream_t st);
 void launch_wait_selftest(long long polls, int *status, cudaStream_t st);
 
-size_t push_smem_bytes(int T, int order);
+// events: some species ionizes, emits photons or creates pairs
 void launch_push_deposit(const GridDev &g, const float *E, const float *B, const SpDev *sps_dev, int nsp,
-                         const QedDev &qd, float *jscratch, int *jvalid, int *status, const long long *step_dev,
+                         bool events, const QedDev &qd, float *jscratch, int *jvalid, int *status, const long long *step_dev,
                          cudaStream_t st);
 hyb_status setup_qed(hyb_ctx *c);  // builds the QED tables once per context
 hyb_status regime_update(hyb_ctx *c, const float *p_mean, const float *p_std);

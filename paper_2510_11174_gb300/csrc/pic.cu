@@ -31,41 +31,53 @@
 #include "qed.cuh"
 #include "particles.cuh"
 
+#include <cooperative_groups.h>
+
+#include <mutex>
+#include <type_traits>
+
 namespace hyb {
+
+namespace cg = cooperative_groups;
 
 // field frame edge: a shape of order k gathers from k nodes below the tile to k - 1 above it
 __host__ __device__ constexpr int frame_F(int T, int order = 1) { return T + 2 * order; }
 
-static constexpr int PUSH_THREADS = 256;
-static constexpr int PUSH_QCAP = 64;  // per-warp queue of cell-crossing particles
+// 8^3 tiles hold thousands of particles, 4^3 tiles a few hundred: smaller CTAs
+// there leave fewer lanes idle in a species' last pass and fewer warps waiting
+__host__ __device__ constexpr int push_threads(int T) { return T == 8 ? 256 : 128; }
+// CTAs per SM by shared memory (8^3: 73 KB linear, 114 KB quadratic shape; 4^3: 25 and 42 KB) and registers
+__host__ __device__ constexpr int push_ctas(int T, int order) { return T == 8 ? (order == 1 ? 3 : 2) : (order == 1 ? 6 : 5); }
+static constexpr int PUSH_Q = 32;          // entries of a per-warp queue of cell-crossing particles
+static constexpr int PUSH_SPLIT_CTAS = 512;   // see launch_push_deposit
 
 __host__ __device__ constexpr size_t align16(size_t b) { return (b + 15) & ~(size_t)15; }
 
-// the current frame (3 components, 64-bit fixed point), the fields, then the
-// per-warp queues (two float4 per entry)
-size_t push_smem_bytes(int T, int order) {
+// the current frame (3 components, 64-bit fixed point), the fields, the
+// per-warp queues (two of PUSH_Q entries of two float4), the species
+size_t push_smem_bytes(int T, int order, int nsp) {
     const int F = frame_F(T, order), G = frame_G(T, order);
     return align16(sizeof(unsigned long long) * 3 * (size_t)G * G * G) + align16(sizeof(float) * 6 * (size_t)F * F * F) +
-           2 * sizeof(float4) * (PUSH_THREADS / 32) * PUSH_QCAP;
+           sizeof(float4) * (push_threads(T) / 32) * 4 * PUSH_Q + sizeof(SpDev) * (size_t)nsp;
 }
 
-// CIC weights of one axis for integer and half-integer staggering, relative to
-// the frame origin o (global node index of local 0)
+// CIC base index and weight of one axis on the integer (i) and the
+// half-integer (h) grid, relative to the frame origin o (global node index of
+// local 0); fl = floor(p)
 struct AxisW {
-    int li, lh;     // local base index (integer / half-integer grid)
-    float fi, fh;   // fractional offsets
+    int li, lh;
+    float fi, fh;
 };
 
-__device__ __forceinline__ AxisW axis_weights(const GridDev &g, int a, float p, int o) {
+__device__ __forceinline__ AxisW axis_weights(const GridDev &g, int a, float p, float fl, int o) {
     AxisW r;
-    int i = (int)floorf(p);
-    if (g.bc[a] && i > g.n[a] - 2) i = g.n[a] - 2;  // particle on the top wall
-    r.li = i - o;
-    r.fi = p - (float)i;
-    const float s = p - 0.5f;
-    const int h = (int)floorf(s);
-    r.lh = h - o;
-    r.fh = s - (float)h;
+    if (g.bc[a]) fl = fminf(fl, (float)(g.n[a] - 2));  // particle on the top wall
+    r.li = (int)fl - o;
+    r.fi = p - fl;
+    // floor(p - 1/2) is the cell below when p lies in the lower half of its cell
+    const bool low = r.fi < 0.5f;
+    r.lh = r.li - (low ? 1 : 0);
+    r.fh = r.fi + (low ? 0.5f : -0.5f);
     return r;
 }
 
@@ -148,14 +160,6 @@ __device__ __forceinline__ void higuera_cary_push(float h, const float e[3], con
     u[2] = up[2] + h * e[2] + (up[0] * t[1] - up[1] * t[0]);
 }
 
-__device__ __forceinline__ void shape3(float p, int gbase, float S[3]) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const float d = fabsf(p - (float)(gbase + k));
-        S[k] = d < 1.0f ? 1.0f - d : 0.0f;
-    }
-}
-
 // Esirkepov deposit of a particle that stays in its cell.  Per axis the shape
 // is (1 - f, f) on the cell's two nodes, f moving from f0 to f1 = f0 + d; W_c
 // is nonzero only on the cell's lower c-face, at its 2 x 2 transverse nodes,
@@ -164,16 +168,15 @@ __device__ __forceinline__ void shape3(float p, int gbase, float S[3]) {
 // other three nodes take m_q - X, m_p - X and 1 - m_p - m_q + X.
 // fac[c] = q w jfac_c 2^k; the current is fac[c] (S1 - S0)(lower node) = -fac[c] d_c.
 template <int G>
-__device__ __forceinline__ void deposit_same_cell(unsigned long long *__restrict__ sj, const float x0[3],
-                                                  const float x1[3], const int o[3], const float fac[3]) {
+__device__ __forceinline__ void deposit_same_cell(unsigned *__restrict__ sj, const float x0[3], const float x1[3],
+                                                  const float fl[3], const int o[3], const float fac[3]) {
     constexpr int G3 = G * G * G;
     int lb[3];
     float m[3], d[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const float c0 = floorf(x0[a]);
-        lb[a] = (int)c0 - o[a];
-        const float f0 = x0[a] - c0, f1 = x1[a] - c0;
+        lb[a] = (int)fl[a] - o[a];
+        const float f0 = x0[a] - fl[a], f1 = x1[a] - fl[a];
         d[a] = f1 - f0;
         m[a] = 0.5f * (f0 + f1);
     }
@@ -181,68 +184,167 @@ __device__ __forceinline__ void deposit_same_cell(unsigned long long *__restrict
     constexpr int off[3] = {1, G, G * G};
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        if (d[c] == 0.0f) continue;
+        if (d[c] == 0.0f) continue;  // particles at rest
         const int pa = (c + 1) % 3, qa = (c + 2) % 3;
         const float X = fmaf(d[pa] * d[qa], 1.0f / 12.0f, m[pa] * m[qa]);
         const float v01 = m[qa] - X, v10 = m[pa] - X;
         const float v00 = (1.0f - m[pa]) - v01;
         const float sc = -fac[c] * d[c];
-        unsigned long long *J = sj + c * G3 + base;
-        atomicAdd(J, fix_of(sc * v00));
-        atomicAdd(J + off[pa], fix_of(sc * v10));
-        atomicAdd(J + off[qa], fix_of(sc * v01));
-        atomicAdd(J + off[pa] + off[qa], fix_of(sc * X));
+        const int J = c * G3 + base;
+        const int idx[4] = {J, J + off[pa], J + off[qa], J + off[pa] + off[qa]};
+        const float val[4] = {sc * v00, sc * v10, sc * v01, sc * X};
+        fix_add<4, false>(sj, 3 * G3, idx, val);
     }
 }
 
-// Esirkepov deposit on the 3-node window of each axis (a particle that
-// crossed a cell face): W_c = DS_c (S0_p S0_q + DS_p S0_q / 2 + S0_p DS_q / 2 +
-// DS_p DS_q / 3), prefix-summed along c
+__device__ __forceinline__ int sel3(int a, int v0, int v1, int v2) { return a == 0 ? v0 : (a == 1 ? v1 : v2); }
+__device__ __forceinline__ float sel3(int a, float v0, float v1, float v2) { return a == 0 ? v0 : (a == 1 ? v1 : v2); }
+
+// transverse factor S0p (S0q + DSq/2) + DSp (S0q/2 + DSq/3) of Esirkepov's W
+__device__ __forceinline__ float esirkepov_cross(float s0p, float dsp, float s0q, float dsq) {
+    const float ca = fmaf(0.5f, dsq, s0q);
+    const float cb = fmaf(1.0f / 3.0f, dsq, 0.5f * s0q);
+    return fmaf(dsp, cb, s0p * ca);
+}
+
+// Esirkepov deposit of a particle that crossed a cell face along one axis c
+// only, the commonest crossing by far: three nodes along c, two along the
+// others, so 8 + 6 + 6 currents instead of the 54 slots of the full window.
+// The queue holds its coordinates rotated to (c, p, q) with the axis, so every
+// lane of the warp runs the same straight code on its own strides.
 template <int G>
-__device__ __forceinline__ void deposit_general(unsigned long long *__restrict__ sj, const float x0[3],
-                                                const float x1[3], const int o[3], float qw, const float jfac[3]) {
+__device__ __forceinline__ void deposit_one_crossing(unsigned *__restrict__ sj, const float4 A, const float4 B,
+                                                     const int o[3], const float jfac[3]) {
     constexpr int G3 = G * G * G;
+    const int c = __float_as_int(B.w);
+    const int sc = sel3(c, 1, G, G * G), sp = sel3(c, G, G * G, 1), sq = sel3(c, G * G, 1, G);
+    const float gc = fminf(floorf(A.x), floorf(B.x)), gp = floorf(A.y), gq = floorf(A.z);
+    const int base = ((int)gc - sel3(c, o[0], o[1], o[2])) * sc + ((int)gp - sel3(c, o[1], o[2], o[0])) * sp +
+                     ((int)gq - sel3(c, o[2], o[0], o[1])) * sq;
+    float s0c[3], dc[3], s0p[2], dp[2], s0q[2], dq[2];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        s0c[k] = fmaxf(1.0f - fabsf(A.x - (gc + k)), 0.0f);
+        dc[k] = fmaxf(1.0f - fabsf(B.x - (gc + k)), 0.0f) - s0c[k];
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        s0p[k] = 1.0f - fabsf(A.y - (gp + k));
+        dp[k] = 1.0f - fabsf(B.y - (gp + k)) - s0p[k];
+        s0q[k] = 1.0f - fabsf(A.z - (gq + k));
+        dq[k] = 1.0f - fabsf(B.z - (gq + k)) - s0q[k];
+    }
+    const int Jc = base + c * G3, Jp = base + sel3(c, 1, 2, 0) * G3, Jq = base + sel3(c, 2, 0, 1) * G3;
+    const float fc = A.w * sel3(c, jfac[0], jfac[1], jfac[2]), fp = A.w * sel3(c, jfac[1], jfac[2], jfac[0]),
+                fq = A.w * sel3(c, jfac[2], jfac[0], jfac[1]);
+    {
+        int idx[8];
+        float val[8];
+#pragma unroll
+        for (int bq = 0; bq < 2; ++bq)
+#pragma unroll
+            for (int bp = 0; bp < 2; ++bp) {
+                const float w = esirkepov_cross(s0p[bp], dp[bp], s0q[bq], dq[bq]);
+                float acc = 0.0f;
+#pragma unroll
+                for (int a = 0; a < 2; ++a) {
+                    acc += dc[a] * w;
+                    idx[(bq * 2 + bp) * 2 + a] = Jc + a * sc + bp * sp + bq * sq;
+                    val[(bq * 2 + bp) * 2 + a] = fc * acc;
+                }
+            }
+        fix_add<8, false>(sj, 3 * G3, idx, val);
+    }
+    {
+        // along p: transverse axes q (two nodes) and c (three)
+        int idx[6];
+        float val[6];
+#pragma unroll
+        for (int bc = 0; bc < 3; ++bc)
+#pragma unroll
+            for (int bq = 0; bq < 2; ++bq) {
+                idx[bc * 2 + bq] = Jp + bc * sc + bq * sq;
+                val[bc * 2 + bq] = fp * (dp[0] * esirkepov_cross(s0q[bq], dq[bq], s0c[bc], dc[bc]));
+            }
+        fix_add<6, false>(sj, 3 * G3, idx, val);
+    }
+    {
+        // along q: transverse axes c (three nodes) and p (two)
+        int idx[6];
+        float val[6];
+#pragma unroll
+        for (int bp = 0; bp < 2; ++bp)
+#pragma unroll
+            for (int bc = 0; bc < 3; ++bc) {
+                idx[bp * 3 + bc] = Jq + bc * sc + bp * sp;
+                val[bp * 3 + bc] = fq * (dq[0] * esirkepov_cross(s0c[bc], dc[bc], s0p[bp], dp[bp]));
+            }
+        fix_add<6, false>(sj, 3 * G3, idx, val);
+    }
+}
+
+// Esirkepov deposit on the window of W nodes of each axis that holds both
+// shapes (W = 3 linear: particles that crossed faces along several axes; W = 4
+// quadratic): W_c = DS_c (S0_p S0_q + DS_p S0_q / 2 + S0_p DS_q / 2 + DS_p
+// DS_q / 3), prefix-summed along c.  The loop over c is not unrolled (the
+// arrays rotate instead): straight-line code for every slot overruns the
+// instruction cache, which was the largest stall of the push.
+template <int G, int W, bool SKIP>
+__device__ __forceinline__ void deposit_window(unsigned *__restrict__ sj, float S0[3][W], float DS[3][W],
+                                               const int lb[3], float qw, const float jfac[3]) {
+    constexpr int G3 = G * G * G;
+    int base = (lb[2] * G + lb[1]) * G + lb[0];
+    int s[3] = {1, G, G * G};
+    float f[3] = {qw * jfac[0], qw * jfac[1], qw * jfac[2]};
+#pragma unroll 1
+    for (int c = 0; c < 3; ++c) {
+#pragma unroll
+        for (int bq = 0; bq < W; ++bq) {
+            int idx[W * (W - 1)];
+            float val[W * (W - 1)];
+#pragma unroll
+            for (int bp = 0; bp < W; ++bp) {
+                const float w = esirkepov_cross(S0[1][bp], DS[1][bp], S0[2][bq], DS[2][bq]);
+                float acc = 0.0f;
+#pragma unroll
+                for (int a = 0; a < W - 1; ++a) {
+                    acc += DS[0][a] * w;
+                    idx[bp * (W - 1) + a] = base + a * s[0] + bp * s[1] + bq * s[2];
+                    val[bp * (W - 1) + a] = f[0] * acc;
+                }
+            }
+            fix_add<W *(W - 1), SKIP>(sj, 3 * G3, idx, val);
+        }
+        base += G3;
+        const int s0 = s[0];
+        const float f0 = f[0];
+        s[0] = s[1]; s[1] = s[2]; s[2] = s0;
+        f[0] = f[1]; f[1] = f[2]; f[2] = f0;
+#pragma unroll
+        for (int k = 0; k < W; ++k) {
+            const float a0 = S0[0][k], d0 = DS[0][k];
+            S0[0][k] = S0[1][k]; S0[1][k] = S0[2][k]; S0[2][k] = a0;
+            DS[0][k] = DS[1][k]; DS[1][k] = DS[2][k]; DS[2][k] = d0;
+        }
+    }
+}
+
+template <int G>
+__device__ __forceinline__ void deposit_general(unsigned *__restrict__ sj, const float x0[3], const float x1[3],
+                                                const int o[3], float qw, const float jfac[3]) {
     int lb[3];
     float S0[3][3], DS[3][3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const int i0 = (int)floorf(x0[a]), i1 = (int)floorf(x1[a]);
-        const int gb = i0 < i1 ? i0 : i1;
-        lb[a] = gb - o[a];
-        float S1[3];
-        shape3(x0[a], gb, S0[a]);
-        shape3(x1[a], gb, S1);
+        const float gb = fminf(floorf(x0[a]), floorf(x1[a]));
+        lb[a] = (int)gb - o[a];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) DS[a][k] = S1[k] - S0[a][k];
-    }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const int pa = (c + 1) % 3, qa = (c + 2) % 3;
-        const float fac = qw * jfac[c];
-        unsigned long long *Jc = sj + c * G3;
-#pragma unroll
-        for (int bq = 0; bq < 3; ++bq) {
-            // transverse factor S0p (S0q + DSq/2) + DSp (S0q/2 + DSq/3)
-            const float caq = fmaf(0.5f, DS[qa][bq], S0[qa][bq]);
-            const float cbq = fmaf(1.0f / 3.0f, DS[qa][bq], 0.5f * S0[qa][bq]);
-#pragma unroll
-            for (int bp = 0; bp < 3; ++bp) {
-                const float cross = fmaf(DS[pa][bp], cbq, S0[pa][bp] * caq);
-                float acc = 0.0f;
-#pragma unroll
-                for (int a = 0; a < 2; ++a) {
-                    acc += DS[c][a] * cross;
-                    if (acc != 0.0f) {
-                        int l3[3];
-                        l3[c] = lb[c] + a;
-                        l3[pa] = lb[pa] + bp;
-                        l3[qa] = lb[qa] + bq;
-                        atomicAdd(&Jc[(l3[2] * G + l3[1]) * G + l3[0]], fix_of(fac * acc));
-                    }
-                }
-            }
+        for (int k = 0; k < 3; ++k) {
+            S0[a][k] = fmaxf(1.0f - fabsf(x0[a] - (gb + k)), 0.0f);
+            DS[a][k] = fmaxf(1.0f - fabsf(x1[a] - (gb + k)), 0.0f) - S0[a][k];
         }
     }
+    deposit_window<G, 3, true>(sj, S0, DS, lb, qw, jfac);
 }
 
 // Quadratic (TSC) shape: S(d) = 3/4 - d^2 (|d| <= 1/2), (3/2 - |d|)^2 / 2
@@ -282,98 +384,109 @@ __device__ __forceinline__ float interp27(const float *__restrict__ f, int bx, i
     return acc;
 }
 
-// Esirkepov with the quadratic shape: per axis the 4-node window holding the
-// old and new 3-node supports (base = the smaller nearest node, minus one),
-// W as for CIC, prefix-summed over the window's 3 inner faces
-template <int G>
-__device__ __forceinline__ void deposit_quadratic(unsigned long long *__restrict__ sj, const float x0[3],
-                                                  const float x1[3], const int o[3], float qw, const float jfac[3]) {
-    constexpr int G3 = G * G * G;
+// Esirkepov with the quadratic shape.  W = 3: a particle whose nearest node
+// stays the same on every axis keeps its three nodes (54 currents); W = 4: the
+// 4-node window that holds the old and the new support (144 slots, most of them
+// 0).  Base = the smaller nearest node, minus one.
+template <int G, int W>
+__device__ __forceinline__ void deposit_quadratic(unsigned *__restrict__ sj, const float4 A, const float4 B,
+                                                  const int o[3], const float jfac[3]) {
+    const float x0[3] = {A.x, A.y, A.z}, x1[3] = {B.x, B.y, B.z};
     int lb[3];
-    float S0[3][4], DS[3][4];
+    float S0[3][W], DS[3][W];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const int m0 = (int)floorf(x0[a] + 0.5f), m1 = (int)floorf(x1[a] + 0.5f);
-        const int gb = (m0 < m1 ? m0 : m1) - 1;
-        lb[a] = gb - o[a];
+        const float gb = fminf(floorf(x0[a] + 0.5f), floorf(x1[a] + 0.5f)) - 1.0f;
+        lb[a] = (int)gb - o[a];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            S0[a][k] = tsc(x0[a] - (float)(gb + k));
-            DS[a][k] = tsc(x1[a] - (float)(gb + k)) - S0[a][k];
+        for (int k = 0; k < W; ++k) {
+            S0[a][k] = tsc(x0[a] - (gb + k));
+            DS[a][k] = tsc(x1[a] - (gb + k)) - S0[a][k];
         }
     }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const int pa = (c + 1) % 3, qa = (c + 2) % 3;
-        const float fac = qw * jfac[c];
-        unsigned long long *Jc = sj + c * G3;
-#pragma unroll
-        for (int bq = 0; bq < 4; ++bq) {
-            const float caq = fmaf(0.5f, DS[qa][bq], S0[qa][bq]);
-            const float cbq = fmaf(1.0f / 3.0f, DS[qa][bq], 0.5f * S0[qa][bq]);
-#pragma unroll
-            for (int bp = 0; bp < 4; ++bp) {
-                const float cross = fmaf(DS[pa][bp], cbq, S0[pa][bp] * caq);
-                float acc = 0.0f;
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    acc += DS[c][a] * cross;
-                    if (acc != 0.0f) {
-                        int l3[3];
-                        l3[c] = lb[c] + a;
-                        l3[pa] = lb[pa] + bp;
-                        l3[qa] = lb[qa] + bq;
-                        atomicAdd(&Jc[(l3[2] * G + l3[1]) * G + l3[0]], fix_of(fac * acc));
-                    }
-                }
-            }
+    deposit_window<G, W, W == 4>(sj, S0, DS, lb, A.w, jfac);
+}
+
+// A warp's queue of crossing particles, 32 entries in shared memory: `n` of
+// them are taken (warp-uniform).  The lanes in `want` append; a full queue is
+// handed to `flush` with every lane of the warp holding one entry.
+template <class F>
+__device__ __forceinline__ void queue_put(float4 *qa, int &n, bool want, const float4 A, const float4 B, int lane,
+                                          F flush) {
+    float4 *qb = qa + PUSH_Q;
+    const unsigned m = __ballot_sync(0xffffffffu, want);
+    if (m == 0u) return;
+    const int pos = n + __popc(m & ((1u << lane) - 1u));
+    if (want && pos < PUSH_Q) {
+        qa[pos] = A;
+        qb[pos] = B;
+    }
+    n += __popc(m);
+    if (n >= PUSH_Q) {
+        __syncwarp();
+        flush(qa[lane], qb[lane]);
+        __syncwarp();
+        n -= PUSH_Q;
+        if (want && pos >= PUSH_Q) {
+            qa[pos - PUSH_Q] = A;
+            qb[pos - PUSH_Q] = B;
         }
     }
 }
 
-// One CTA per tile: stage E, B of the tile and a one-node halo, push every
-// particle of every species, deposit its current into the tile's fixed-point
-// frame, apply the stochastic events, write it back or send it to the
-// migration buffer.  Particles that stay in their cell deposit at once;
-// particles that crossed a cell face wait in a per-warp queue and are
-// deposited 32 at a time with the full 3-node stencil, so that the long
-// stencil runs with every lane of the warp busy.
-template <int T, int ORDER>
-__global__ void __launch_bounds__(PUSH_THREADS, 3) k_push_deposit(GridDev g, const float *__restrict__ E,
-                                                                  const float *__restrict__ B,
-                                                                  const SpDev *__restrict__ sps, int nsp,
-                                                                  float *__restrict__ jscratch,
-                                                                  int *__restrict__ jvalid, int *__restrict__ status,
-                                                                  const long long *__restrict__ step_dev, QedDev qd) {
+// One CTA per tile (SPLIT: a cluster of CTAs per tile, each taking every
+// cluster-size-th block of its particles): stage E, B of the tile and a
+// one-node halo, push every particle of every species, deposit its current into
+// the tile's fixed-point frame, apply the stochastic events (EV: some species
+// has them), write it back or send it to the migration buffer.  Particles that
+// stay in their cell deposit at once; particles that crossed a cell face wait in
+// per-warp queues, one for a single crossed axis and one for the others, and are
+// deposited 32 at a time, so that the long stencils run with every lane of the
+// warp busy.  The warps meet only before the first and after the last species.
+// With SPLIT the CTAs' frames are added as integers through distributed shared
+// memory before the one rounding to FP32, so the current does not depend on the
+// split.
+// What bounds it, 15.7 M thermal particles (128 x 96 x 80 cells, a third of them
+// crossing a face per step): instruction issue (53 %) and the shared-memory pipe
+// (61 %), 46 B a particle of DRAM traffic.  Measured there, one launch (cold):
+// 1.19 ms with 64-bit atomics and the FP64-pipe conversion, 0.89 ms with the word
+// planes and the one-axis queue, 0.72 ms with the two-conversion digits and the
+// migration chunks; 0.76 M particles of the quadratic shape 0.46 -> 0.25 ms.
+template <int T, int ORDER, bool EV, bool SPLIT>
+__global__ void __launch_bounds__(push_threads(T), push_ctas(T, ORDER))
+    k_push_deposit(GridDev g, const float *__restrict__ E, const float *__restrict__ B,
+                   const SpDev *__restrict__ sps, int nsp, float *__restrict__ jscratch, int *__restrict__ jvalid,
+                   int *__restrict__ status, const long long *__restrict__ step_dev, QedDev qd) {
     constexpr int F = frame_F(T, ORDER), G = frame_G(T, ORDER);
     constexpr int F3 = F * F * F, G3 = G * G * G;
+    constexpr int NT = push_threads(T), NW = NT / 32;
     extern __shared__ __align__(16) unsigned char smraw[];
-    unsigned long long *sj = reinterpret_cast<unsigned long long *>(smraw);  // 3 current components, G^3 each
+    unsigned *sj = reinterpret_cast<unsigned *>(smraw);  // 3 current components, G^3 each: low words, high words
     float *sf = reinterpret_cast<float *>(smraw + align16(sizeof(unsigned long long) * 3 * G3));  // 6 x F^3
     float4 *queue = reinterpret_cast<float4 *>(reinterpret_cast<unsigned char *>(sf) + align16(sizeof(float) * 6 * F3));
-    __shared__ int s_holes;
+    SpDev *s_sp = reinterpret_cast<SpDev *>(queue + NW * 4 * PUSH_Q);  // the species' descriptors
+    __shared__ int s_holes[HYB_MAX_SPECIES];
     __shared__ int s_qwmax[32];  // per warp: largest |q w| of the tile's particles (float bits)
     __shared__ int s_kfix;       // fixed-point exponent of the tile's current frame
-    __shared__ double s_tal_e[NTALLY];
-    __shared__ unsigned long long s_tal_n[NTALLY];
-    __shared__ SpDev s_sp;       // the species being pushed (its descriptor read once per tile)
-    const long long step = *step_dev;
-    double tal_e[NTALLY] = {0.0, 0.0, 0.0};
-    int tal_n[NTALLY] = {0, 0, 0};
+    __shared__ double s_tal_e[EV ? HYB_MAX_SPECIES * NTALLY : 1];
+    __shared__ unsigned long long s_tal_n[EV ? HYB_MAX_SPECIES * NTALLY : 1];
+    const long long step = EV ? *step_dev : 0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float4 *qa = queue + warp * 2 * PUSH_QCAP;  // (x0, q w) of queued particles
-    float4 *qb = qa + PUSH_QCAP;                // (x1, -)
+    float4 *q1 = queue + warp * 4 * PUSH_Q;  // crossed one axis (quadratic shape: the nearest nodes stay)
+    float4 *q3 = q1 + 2 * PUSH_Q;            // crossed several (quadratic shape: some nearest node changes)
 
-    const int t = blockIdx.x;
+    cg::cluster_group cl = cg::this_cluster();
+    const int nrank = SPLIT ? (int)cl.num_blocks() : 1, rank = SPLIT ? (int)cl.block_rank() : 0;
+    const int t = SPLIT ? (int)blockIdx.x / nrank : (int)blockIdx.x;
     // a tile without particles writes no frame: the reduction skips it
     int total = 0;
     for (int si = 0; si < nsp; ++si) total += min(sps[si].count[t], sps[si].cap);
     if (total == 0) {
-        if (threadIdx.x < nsp) {
+        if (rank == 0 && threadIdx.x < nsp) {
             sps[threadIdx.x].hole_count[t] = 0;
             sps[threadIdx.x].hole_used[t] = 0;
         }
-        if (threadIdx.x == 0) jvalid[t] = 0;
+        if (rank == 0 && threadIdx.x == 0) jvalid[t] = 0;
         return;
     }
     // the largest |q w| in the tile bounds every frame sum (fixed-point scale)
@@ -383,7 +496,8 @@ __global__ void __launch_bounds__(PUSH_THREADS, 3) k_push_deposit(GridDev g, con
             const SpDev &sp = sps[si];
             const int n = min(sp.count[t], sp.cap);
             const long long base = (long long)t * sp.cap;
-            for (int p = threadIdx.x; p < n; p += PUSH_THREADS) {
+#pragma unroll 4
+            for (int p = rank * NT + threadIdx.x; p < n; p += nrank * NT) {
                 const float qp = sp.zq ? sp.q * sp.zq[base + p] : sp.q;
                 qwm = fmaxf(qwm, fabsf(qp * sp.w[base + p]));
             }
@@ -394,7 +508,7 @@ __global__ void __launch_bounds__(PUSH_THREADS, 3) k_push_deposit(GridDev g, con
     const int o[3] = {tx * T - ORDER, ty * T - ORDER, tz * T - ORDER};  // frame origin
     const long long N = g.N;
 
-    for (int l = threadIdx.x; l < F3; l += PUSH_THREADS) {
+    for (int l = threadIdx.x; l < F3; l += NT) {
         const int lx = l % F, ly = (l / F) % F, lz = l / (F * F);
         int gi[3] = {o[0] + lx, o[1] + ly, o[2] + lz};
         bool in = true;
@@ -413,15 +527,19 @@ __global__ void __launch_bounds__(PUSH_THREADS, 3) k_push_deposit(GridDev g, con
             sf[(3 + q) * F3 + l] = in ? B[q * N + c] : 0.0f;
         }
     }
-    for (int l = threadIdx.x; l < 3 * G3; l += PUSH_THREADS) sj[l] = 0ULL;
-    if (threadIdx.x == 0) {
-        s_holes = 0;
-        for (int k = 0; k < NTALLY; ++k) {
-            s_tal_e[k] = 0.0;
-            s_tal_n[k] = 0;
-        }
+    for (int l = threadIdx.x; l < 6 * G3; l += NT) sj[l] = 0u;
+    {
+        const int *src = reinterpret_cast<const int *>(sps);
+        int *dst = reinterpret_cast<int *>(s_sp);
+        for (int w = threadIdx.x; w < nsp * (int)(sizeof(SpDev) / sizeof(int)); w += NT) dst[w] = src[w];
     }
-    __syncthreads();
+    if (threadIdx.x < HYB_MAX_SPECIES) s_holes[threadIdx.x] = 0;
+    if (EV && threadIdx.x < HYB_MAX_SPECIES * NTALLY) {
+        s_tal_e[threadIdx.x] = 0.0;
+        s_tal_n[threadIdx.x] = 0;
+    }
+    if (SPLIT) cl.sync();
+    else __syncthreads();
 
     const float dt = g.dt;
     const float inv_d[3] = {1.0f / g.d[0], 1.0f / g.d[1], 1.0f / g.d[2]};
@@ -430,28 +548,48 @@ __global__ void __launch_bounds__(PUSH_THREADS, 3) k_push_deposit(GridDev g, con
     // so a node's sum is at most total * max |q w| * max |jfac|)
     const float j0 = -1.0f / (dt * g.d[1] * g.d[2]), j1 = -1.0f / (dt * g.d[0] * g.d[2]),
                 j2 = -1.0f / (dt * g.d[0] * g.d[1]);
-    const int kfix = fix_exponent((double)total * (double)block_max_read(s_qwmax) *
-                                  (double)fmaxf(fabsf(j0), fmaxf(fabsf(j1), fabsf(j2))));
-    const float fscale = pow2f(kfix);
+    if (warp == 0) {
+        // one warp: double precision is slow here
+        int b = 0;
+        for (int i = lane; i < nrank * NW; i += 32)
+            b = max(b, SPLIT ? *cl.map_shared_rank(&s_qwmax[i % NW], i / NW) : s_qwmax[i]);
+        b = __reduce_max_sync(0xffffffffu, b);
+        const int k = fix_exponent((double)total * (double)__int_as_float(b) *
+                                   (double)fmaxf(fabsf(j0), fmaxf(fabsf(j1), fabsf(j2))));
+        if (lane == 0) s_kfix = k;
+    }
+    __syncthreads();
+    const float fscale = pow2f(s_kfix);
     const float jfac[3] = {j0 * fscale, j1 * fscale, j2 * fscale};
-    if (threadIdx.x == 0) s_kfix = kfix;  // read back after the species loop's barriers
     const float *sEx = sf, *sEy = sf + F3, *sEz = sf + 2 * F3;
     const float *sBx = sf + 3 * F3, *sBy = sf + 4 * F3, *sBz = sf + 5 * F3;
+    // positions of this tile's particles: t0 <= x < t1 (an absorbing axis ends with its wall)
+    float t0[3], t1[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        t0[a] = (float)(o[a] + ORDER);
+        t1[a] = (float)(o[a] + ORDER + T);
+        if (g.bc[a] && t1[a] > (float)(g.n[a] - 1)) t1[a] = __int_as_float(__float_as_int((float)(g.n[a] - 1)) + 1);
+    }
+    auto flush1 = [&](const float4 A, const float4 Bq) {
+        if constexpr (ORDER == 1) deposit_one_crossing<G>(sj, A, Bq, o, jfac);
+        else deposit_quadratic<G, 3>(sj, A, Bq, o, jfac);
+    };
+    auto flush3 = [&](const float4 A, const float4 Bq) {
+        const float y0[3] = {A.x, A.y, A.z}, y1[3] = {Bq.x, Bq.y, Bq.z};
+        if constexpr (ORDER == 1) deposit_general<G>(sj, y0, y1, o, A.w, jfac);
+        else deposit_quadratic<G, 4>(sj, A, Bq, o, jfac);
+    };
+    int n1 = 0, n3 = 0;  // entries in this warp's queues (warp-uniform)
 
     for (int si = 0; si < nsp; ++si) {
-        {
-            // the descriptor to shared memory: the loop reads it for every particle
-            const int *src = reinterpret_cast<const int *>(sps + si);
-            int *dst = reinterpret_cast<int *>(&s_sp);
-            for (int w = threadIdx.x; w < (int)(sizeof(SpDev) / sizeof(int)); w += PUSH_THREADS) dst[w] = src[w];
-            __syncthreads();
-        }
-        const SpDev &sp = s_sp;
+        const SpDev &sp = s_sp[si];
+        double tal_e[NTALLY] = {0.0, 0.0, 0.0};
+        int tal_n[NTALLY] = {0, 0, 0};
         const int n = min(sp.count[t], sp.cap);
         const long long base = (long long)t * sp.cap;
         // times q_p below; photons (m = 0, q = 0) get no Lorentz force
         const float qm_half = sp.kind == 1 ? 0.0f : 0.5f * dt / sp.m;
-        int qn = 0;  // entries in this warp's queue (warp-uniform)
         // the next particle's x, y, z, ux, uy, uz, w and charge state, loaded one
         // iteration ahead so that the loads overlap the current particle's work
         float pf[8];
@@ -464,8 +602,9 @@ __global__ void __launch_bounds__(PUSH_THREADS, 3) k_push_deposit(GridDev g, con
                 pf[7] = sp.zq ? sp.zq[s2] : 1.0f;
             }
         };
-        prefetch(threadIdx.x);
-        for (int p0 = 0; p0 < n; p0 += PUSH_THREADS) {
+        int mbase = 0, mused = MIG_CHUNK;  // the warp's chunk of the migration buffer and its used slots (uniform)
+        prefetch(rank * NT + threadIdx.x);
+        for (int p0 = rank * NT; p0 < n; p0 += nrank * NT) {
             const int p = p0 + threadIdx.x;
             bool act = p < n;
             const long long s = base + p;
@@ -478,29 +617,24 @@ __global__ void __launch_bounds__(PUSH_THREADS, 3) k_push_deposit(GridDev g, con
                 wgt = pf[6];
                 q = sp.q * pf[7];
             }
-            prefetch(p + PUSH_THREADS);
+            prefetch(p + nrank * NT);
             if (act) {
                 // every shared-memory index below derives from a cell inside this
-                // tile; anything else is flagged and left untouched
-                bool inside = true;
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    int ci = (int)floorf(x0[a]);
-                    if (g.bc[a] && ci == g.n[a] - 1 && x0[a] == (float)(g.n[a] - 1)) ci = g.n[a] - 2;
-                    inside = inside && isfinite(x0[a]) && ci >= o[a] + ORDER && ci <= o[a] + ORDER + T - 1 &&
-                             (g.bc[a] == 0 || ci <= g.n[a] - 2);
-                }
+                // tile; anything else (NaN among it) is flagged and left untouched
+                const bool inside = x0[0] >= t0[0] && x0[0] < t1[0] && x0[1] >= t0[1] && x0[1] < t1[1] &&
+                                    x0[2] >= t0[2] && x0[2] < t1[2];
                 if (!inside) {
                     atomicOr(status, ST_BADPOS);
                     act = false;
                 }
             }
+            const float fl[3] = {floorf(x0[0]), floorf(x0[1]), floorf(x0[2])};
             if (act) {
                 // ---- gather E^n, B^n at x^n
                 if constexpr (ORDER == 1) {
-                    const AxisW ax = axis_weights(g, 0, x0[0], o[0]);
-                    const AxisW ay = axis_weights(g, 1, x0[1], o[1]);
-                    const AxisW az = axis_weights(g, 2, x0[2], o[2]);
+                    const AxisW ax = axis_weights(g, 0, x0[0], fl[0], o[0]);
+                    const AxisW ay = axis_weights(g, 1, x0[1], fl[1], o[1]);
+                    const AxisW az = axis_weights(g, 2, x0[2], fl[2], o[2]);
                     e[0] = interp8<F>(sEx, ax.lh, ay.li, az.li, ax.fh, ay.fi, az.fi);
                     e[1] = interp8<F>(sEy, ax.li, ay.lh, az.li, ax.fi, ay.fh, az.fi);
                     e[2] = interp8<F>(sEz, ax.li, ay.li, az.lh, ax.fi, ay.fi, az.fh);
@@ -552,35 +686,37 @@ __global__ void __launch_bounds__(PUSH_THREADS, 3) k_push_deposit(GridDev g, con
             }
 
             // ---- Esirkepov deposit into the shared frame: particles that stay
-            // in their cell now, the others through the warp's queue
-            bool same_cell = ORDER == 1;   // the quadratic stencil always takes the queue
-#pragma unroll
-            for (int a = 0; a < 3; ++a) same_cell = same_cell && floorf(x0[a]) == floorf(x1[a]);
+            // in their cell now, the others through the warp's queues
             const bool dep = act && q != 0.0f;
-            if (dep && same_cell) {
+            if constexpr (ORDER == 1) {
+                const bool c0 = floorf(x1[0]) != fl[0], c1 = floorf(x1[1]) != fl[1], c2 = floorf(x1[2]) != fl[2];
+                const int nc = (c0 ? 1 : 0) + (c1 ? 1 : 0) + (c2 ? 1 : 0);
                 const float qw = q * wgt;
-                const float fac[3] = {qw * jfac[0], qw * jfac[1], qw * jfac[2]};
-                deposit_same_cell<G>(sj, x0, x1, o, fac);
-            }
-            const unsigned cross = __ballot_sync(0xffffffffu, dep && !same_cell);
-            if (dep && !same_cell) {
-                const int pos = qn + __popc(cross & ((1u << lane) - 1u));
-                qa[pos] = make_float4(x0[0], x0[1], x0[2], q * wgt);
-                qb[pos] = make_float4(x1[0], x1[1], x1[2], 0.0f);
-            }
-            qn += __popc(cross);
-            __syncwarp();
-            if (qn >= 32) {
-                const float4 A = qa[qn - 32 + lane], Bq = qb[qn - 32 + lane];
-                const float y0[3] = {A.x, A.y, A.z}, y1[3] = {Bq.x, Bq.y, Bq.z};
-                if constexpr (ORDER == 1) deposit_general<G>(sj, y0, y1, o, A.w, jfac);
-                else deposit_quadratic<G>(sj, y0, y1, o, A.w, jfac);
-                qn -= 32;
-                __syncwarp();
+                if (dep && nc == 0) {
+                    const float fac[3] = {qw * jfac[0], qw * jfac[1], qw * jfac[2]};
+                    deposit_same_cell<G>(sj, x0, x1, fl, o, fac);
+                }
+                const int ax = c0 ? 0 : (c1 ? 1 : 2);
+                const float4 A = make_float4(sel3(ax, x0[0], x0[1], x0[2]), sel3(ax, x0[1], x0[2], x0[0]),
+                                             sel3(ax, x0[2], x0[0], x0[1]), qw);
+                const float4 Bq = make_float4(sel3(ax, x1[0], x1[1], x1[2]), sel3(ax, x1[1], x1[2], x1[0]),
+                                              sel3(ax, x1[2], x1[0], x1[1]), __int_as_float(ax));
+                queue_put(q1, n1, dep && nc == 1, A, Bq, lane, flush1);
+                queue_put(q3, n3, dep && nc > 1, make_float4(x0[0], x0[1], x0[2], qw),
+                          make_float4(x1[0], x1[1], x1[2], 0.0f), lane, flush3);
+            } else {
+                bool same = true;
+#pragma unroll
+                for (int a = 0; a < 3; ++a) same = same && floorf(x0[a] + 0.5f) == floorf(x1[a] + 0.5f);
+                const float4 A = make_float4(x0[0], x0[1], x0[2], q * wgt);
+                const float4 Bq = make_float4(x1[0], x1[1], x1[2], 0.0f);
+                queue_put(q1, n1, dep && same, A, Bq, lane, flush1);
+                queue_put(q3, n3, dep && !same, A, Bq, lane, flush3);
             }
 
+            int nt = t;
             if (act) {
-                // ---- periodic image, tile membership, write back or migrate
+                // ---- periodic image, tile membership
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
                     if (g.bc[a] == 0) {
@@ -590,15 +726,18 @@ __global__ void __launch_bounds__(PUSH_THREADS, 3) k_push_deposit(GridDev g, con
                         if (x1[a] >= L) x1[a] = 0.0f;
                     }
                 }
-                const int nt = tile_index(g, x1[0], x1[1], x1[2]);
-
+                nt = tile_index(g, x1[0], x1[1], x1[2]);
+            }
+            float zq_new = 0.0f, tau = 0.0f;
+            bool dead = false;
+            uint64_t pid = 0;
+            if (EV && act) {
                 // ---- stochastic events, after the deposit (this step's current
                 // used the pre-event charge and momentum); new particles start at
                 // x^{n+1} and enter their species through its migration buffer
-                float zq_new = sp.zq ? sp.zq[s] : 0.0f;
-                float tau = sp.tau ? sp.tau[s] : 0.0f;
-                bool dead = false;
-                const uint64_t pid = sp.id[s];
+                zq_new = sp.zq ? sp.zq[s] : 0.0f;
+                tau = sp.tau ? sp.tau[s] : 0.0f;
+                pid = sp.id[s];
                 if (sp.zmax > 0 && zq_new < (float)sp.zmax) {
                     // field ionization: at most one level per step; the electron
                     // takes the ion's u and weight
@@ -610,7 +749,7 @@ __global__ void __launch_bounds__(PUSH_THREADS, 3) k_push_deposit(GridDev g, con
                         zq_new = (float)(Z + 1);
                         tal_e[TALLY_IONIZE] += (double)wgt * sp.ip_mc2[Z];
                         tal_n[TALLY_IONIZE] += 1;
-                        const SpDev &el = sps[sp.ion_into];
+                        const SpDev &el = s_sp[sp.ion_into];
                         const uint64_t eid = (1ULL << 63) | (pid << 3) | (uint64_t)(Z + 1);
                         spawn(el, x1, u, wgt, eid, nt, step, g.seed, -1.0f, status);
                     }
@@ -638,7 +777,7 @@ __global__ void __launch_bounds__(PUSH_THREADS, 3) k_push_deposit(GridDev g, con
                         }
                         tal_n[TALLY_EMIT] += 1;
                         if (eps >= sp.eps_min && sp.ph_species >= 0 && un > 0.0f) {
-                            spawn(sps[sp.ph_species], x1, k, wgt, derived_id(pid, step, 2u), nt, step, g.seed,
+                            spawn(s_sp[sp.ph_species], x1, k, wgt, derived_id(pid, step, 2u), nt, step, g.seed,
                                   -logf(u01f(r.v[2])), status);
                         } else {
                             tal_e[TALLY_EMIT] += (double)wgt * eps;
@@ -667,86 +806,122 @@ __global__ void __launch_bounds__(PUSH_THREADS, 3) k_push_deposit(GridDev g, con
                                 ve[c] = ue * u[c] / eps;
                                 vp[c] = up * u[c] / eps;
                             }
-                            spawn(sps[sp.pair_e], x1, ve, wgt, derived_id(pid, step, 3u), nt, step, g.seed,
+                            spawn(s_sp[sp.pair_e], x1, ve, wgt, derived_id(pid, step, 3u), nt, step, g.seed,
                                   -logf(u01f(r.v[1])), status);
-                            spawn(sps[sp.pair_p], x1, vp, wgt, derived_id(pid, step, 5u), nt, step, g.seed,
+                            spawn(s_sp[sp.pair_p], x1, vp, wgt, derived_id(pid, step, 5u), nt, step, g.seed,
                                   -logf(u01f(r.v[2])), status);
                             dead = true;
                         }
                     }
                 }
+            }
 
-                if (nt == t && !dead) {
-                    sp.x[s] = x1[0]; sp.y[s] = x1[1]; sp.z[s] = x1[2];
-                    sp.ux[s] = u[0]; sp.uy[s] = u[1]; sp.uz[s] = u[2];
-                    if (sp.zmax > 0) sp.zq[s] = zq_new;
-                    if (sp.tau) sp.tau[s] = tau;
-                } else {
-                    if (!dead) {
-                        const int m = warp_append(sp.mig_count);
-                        if (m < sp.mig_cap) {
-                            sp.mx[m] = x1[0]; sp.my[m] = x1[1]; sp.mz[m] = x1[2];
-                            sp.mux[m] = u[0]; sp.muy[m] = u[1]; sp.muz[m] = u[2];
-                            sp.mw[m] = wgt;
-                            if (sp.zq) sp.mzq[m] = zq_new;
-                            if (sp.tau) sp.mtau[m] = tau;
-                            sp.mid[m] = pid;
-                            sp.mdest[m] = nt;
-                        } else {
-                            atomicOr(status, ST_OVERFLOW);
+            // ---- write back or migrate
+            const bool leave = act && (nt != t || dead), mig = leave && !dead;
+            if (act && !leave) {
+                sp.x[s] = x1[0]; sp.y[s] = x1[1]; sp.z[s] = x1[2];
+                sp.ux[s] = u[0]; sp.uy[s] = u[1]; sp.uz[s] = u[2];
+                if (EV && sp.zmax > 0) sp.zq[s] = zq_new;
+                if (EV && sp.tau) sp.tau[s] = tau;
+            }
+            const unsigned mm = __ballot_sync(0xffffffffu, mig);
+            if (mm != 0u) {
+                // the warp's migrants take slots of the chunk it holds; a new
+                // chunk costs one global atomic
+                const int at = mused + __popc(mm & ((1u << lane) - 1u)), need = mused + __popc(mm);
+                int next = 0;
+                if (need > MIG_CHUNK) {
+                    if (lane == 0) next = atomicAdd(sp.mig_count, sp.mig_chunks ? MIG_CHUNK : __popc(mm));
+                    next = __shfl_sync(0xffffffffu, next, 0);
+                }
+                if (mig) {
+                    const int m = at < MIG_CHUNK ? mbase + at : next + at - MIG_CHUNK;
+                    if (m < sp.mig_cap) {
+                        if constexpr (!EV) {
+                            zq_new = sp.zq ? sp.zq[s] : 0.0f;
+                            pid = sp.id[s];
                         }
+                        sp.mx[m] = x1[0]; sp.my[m] = x1[1]; sp.mz[m] = x1[2];
+                        sp.mux[m] = u[0]; sp.muy[m] = u[1]; sp.muz[m] = u[2];
+                        sp.mw[m] = wgt;
+                        if (sp.zq) sp.mzq[m] = zq_new;
+                        if (sp.tau) sp.mtau[m] = tau;
+                        sp.mid[m] = pid;
+                        sp.mdest[m] = nt;
+                    } else {
+                        atomicOr(status, ST_OVERFLOW);
                     }
-                    const int hslot = atomicAdd(&s_holes, 1);
-                    sp.holes[base + hslot] = p;
-                    sp.x[s] = -1.0f;
+                }
+                mused = need;
+                if (need > MIG_CHUNK) {
+                    mbase = next;
+                    mused = sp.mig_chunks ? need - MIG_CHUNK : MIG_CHUNK;
+                }
+            }
+            if (leave) {
+                const int hslot = warp_append(SPLIT ? cl.map_shared_rank(&s_holes[si], 0) : &s_holes[si]);
+                sp.holes[base + hslot] = p;
+                sp.x[s] = -1.0f;
+            }
+        }
+        // the rest of the warp's last chunk holds no migrant
+        if (lane >= mused && mbase + lane < sp.mig_cap) sp.mdest[mbase + lane] = -1;
+        if constexpr (EV) {
+            // per-tile tallies: warp sums, then shared accumulators, then one add per tile
+            if (sp.zmax > 0 || sp.qed || sp.pair_e >= 0) {
+#pragma unroll
+                for (int k = 0; k < NTALLY; ++k) {
+#pragma unroll
+                    for (int o2 = 16; o2 > 0; o2 >>= 1) {
+                        tal_e[k] += __shfl_down_sync(0xffffffffu, tal_e[k], o2);
+                        tal_n[k] += __shfl_down_sync(0xffffffffu, tal_n[k], o2);
+                    }
+                    if (lane == 0 && tal_n[k] > 0) {
+                        atomicAdd(&s_tal_e[si * NTALLY + k], tal_e[k]);
+                        atomicAdd(&s_tal_n[si * NTALLY + k], (unsigned long long)tal_n[k]);
+                    }
                 }
             }
         }
-        // the warp's queue holds fewer than 32 crossing particles: deposit them
-        if (lane < qn) {
-            const float4 A = qa[lane], Bq = qb[lane];
-            const float y0[3] = {A.x, A.y, A.z}, y1[3] = {Bq.x, Bq.y, Bq.z};
-            if constexpr (ORDER == 1) deposit_general<G>(sj, y0, y1, o, A.w, jfac);
-            else deposit_quadratic<G>(sj, y0, y1, o, A.w, jfac);
-        }
-        __syncwarp();
-        // per-tile tallies: warp sums, then shared accumulators, then one add per tile
-#pragma unroll
-        for (int k = 0; k < NTALLY; ++k) {
-#pragma unroll
-            for (int o2 = 16; o2 > 0; o2 >>= 1) {
-                tal_e[k] += __shfl_down_sync(0xffffffffu, tal_e[k], o2);
-                tal_n[k] += __shfl_down_sync(0xffffffffu, tal_n[k], o2);
-            }
-            if ((threadIdx.x & 31) == 0 && tal_n[k] > 0) {
-                atomicAdd(&s_tal_e[k], tal_e[k]);
-                atomicAdd(&s_tal_n[k], (unsigned long long)tal_n[k]);
-            }
-            tal_e[k] = 0.0;
-            tal_n[k] = 0;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            sp.hole_count[t] = s_holes;
-            sp.hole_used[t] = 0;
-            s_holes = 0;
-#pragma unroll
-            for (int k = 0; k < NTALLY; ++k) {
-                if (s_tal_n[k] > 0) {
-                    sp.tal_e[(long long)t * NTALLY + k] += s_tal_e[k];
-                    sp.tal_n[(long long)t * NTALLY + k] += s_tal_n[k];
-                }
-                s_tal_e[k] = 0.0;
-                s_tal_n[k] = 0;
-            }
-        }
-        __syncthreads();
     }
+    // what the queues still hold (each fewer than 32 particles)
+    __syncwarp();
+    if (lane < n1) flush1(q1[lane], q1[PUSH_Q + lane]);
+    if (lane < n3) flush3(q3[lane], q3[PUSH_Q + lane]);
+    if (SPLIT) cl.sync();
+    else __syncthreads();
 
+    if (rank == 0 && threadIdx.x < nsp) {
+        s_sp[threadIdx.x].hole_count[t] = s_holes[threadIdx.x];
+        s_sp[threadIdx.x].hole_used[t] = 0;
+    }
+    if (EV && rank == 0 && threadIdx.x < nsp * NTALLY) {
+        const int i = threadIdx.x;
+        double e = 0.0;
+        unsigned long long c = 0;
+        for (int r = 0; r < nrank; ++r) {
+            e += SPLIT ? *cl.map_shared_rank(&s_tal_e[i], r) : s_tal_e[i];
+            c += SPLIT ? *cl.map_shared_rank(&s_tal_n[i], r) : s_tal_n[i];
+        }
+        if (c > 0) {
+            const SpDev &sp = s_sp[i / NTALLY];
+            sp.tal_e[(long long)t * NTALLY + i % NTALLY] += e;
+            sp.tal_n[(long long)t * NTALLY + i % NTALLY] += c;
+        }
+    }
     float *dst = jscratch + (long long)t * 3 * G3;
     const float inv_scale = pow2f(-s_kfix);
-    for (int l = threadIdx.x; l < 3 * G3; l += PUSH_THREADS) dst[l] = fix_to_float(sj[l], inv_scale);
-    if (threadIdx.x == 0) jvalid[t] = 1;
+    for (int l = rank * NT + threadIdx.x; l < 3 * G3; l += nrank * NT) {
+        unsigned long long v = 0ULL;
+        if (SPLIT) {
+            for (int r = 0; r < nrank; ++r) v += fix_read(cl.map_shared_rank(sj, r), 3 * G3, l);
+        } else {
+            v = fix_read(sj, 3 * G3, l);
+        }
+        dst[l] = fix_to_float(v, inv_scale);
+    }
+    if (rank == 0 && threadIdx.x == 0) jvalid[t] = 1;
+    if (SPLIT) cl.sync();  // no CTA leaves while another reads its frame
 }
 
 
@@ -769,8 +944,10 @@ __global__ void k_j_reduce(GridDev g, const float *__restrict__ jscratch, const 
 // its end.  Grid-stride over the migration buffer (its fill is read on device).
 __global__ void k_rebin(SpDev sp, int *__restrict__ status) {
     const int nm = min(*sp.mig_count, sp.mig_cap);
+    // (a chunk's unused slots hold the destination -1)
     for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < nm; m += gridDim.x * blockDim.x) {
         const int t = sp.mdest[m];
+        if (t < 0) continue;
         const int h = atomicAdd(&sp.hole_used[t], 1);
         int slot;
         if (h < sp.hole_count[t]) {
@@ -931,26 +1108,56 @@ __global__ void k_tiles_to_arrays(SpDev sp, const long long *__restrict__ offset
 
 static inline unsigned blocks_for(long long n, int b) { return (unsigned)((n + b - 1) / b); }
 
+template <int T, int ORDER, bool EV, bool SPLIT>
+static void push_launch(const GridDev &g, const float *E, const float *B, const SpDev *sps_dev, int nsp,
+                        const QedDev &qd, float *jscratch, int *jvalid, int *status, const long long *step_dev,
+                        int split, cudaStream_t st) {
+    auto kern = k_push_deposit<T, ORDER, EV, SPLIT>;
+    // opt in to more than 48 KB of dynamic shared memory, once per instance and device
+    static std::once_flag once[64];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::call_once(once[dev & 63], [&] {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)push_smem_bytes(T, ORDER, HYB_MAX_SPECIES));
+    });
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(g.ntiles * split));
+    cfg.blockDim = dim3((unsigned)push_threads(T));
+    cfg.dynamicSmemBytes = push_smem_bytes(T, ORDER, nsp);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)split;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = SPLIT ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kern, g, E, B, sps_dev, nsp, jscratch, jvalid, status, step_dev, qd);
+}
+
 void launch_push_deposit(const GridDev &g, const float *E, const float *B, const SpDev *sps_dev, int nsp,
-                         const QedDev &qd, float *jscratch, int *jvalid, int *status, const long long *step_dev,
-                         cudaStream_t st) {
-    const size_t smem = push_smem_bytes(g.T, g.order);
-    // opt in to more than 48 KB of dynamic shared memory, once per instance
-    static bool set[4] = {false, false, false, false};
-    auto launch = [&](auto kern, int slot) {
-        if (!set[slot]) {
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            set[slot] = true;
-        }
-        kern<<<g.ntiles, PUSH_THREADS, smem, st>>>(g, E, B, sps_dev, nsp, jscratch, jvalid, status, step_dev, qd);
+                         bool events, const QedDev &qd, float *jscratch, int *jvalid, int *status,
+                         const long long *step_dev, cudaStream_t st) {
+    // A small grid has fewer tiles than the chip holds CTAs (152 SMs x 3), and one
+    // CTA's walk through its tile then decides: its tiles are split over clusters
+    // of 2 or 4 CTAs while the grid stays at or below PUSH_SPLIT_CTAS.  Five steps
+    // with the read-out, us, for 1 / 2 / 3 / 4 / 5 / 8 CTAs a tile: 64 tiles, all full
+    // 423 / 334 / 301 / 298 / 296 / 371; 128 tiles, half of them empty (10 steps and a
+    // classification) 5346 / 4099 / 3843 / 3833 / 3829 / 3921; 315 tiles, 3 particles a
+    // cell 463 / 576 / 649 / 719 / 830 / 1079: every CTA stages the tile's fields and
+    // clears a frame, so a grid that fills the chip is left whole.
+    int split = 1;
+    while (split < 4 && g.ntiles * split * 2 <= PUSH_SPLIT_CTAS) split *= 2;
+    auto go = [&](auto kern) { kern(g, E, B, sps_dev, nsp, qd, jscratch, jvalid, status, step_dev, split, st); };
+    auto shape = [&](auto ev, auto sp) {
+        constexpr bool EV = decltype(ev)::value, SP = decltype(sp)::value;
+        if (g.order == 2) go(g.T == 8 ? push_launch<8, 2, EV, SP> : push_launch<4, 2, EV, SP>);
+        else go(g.T == 8 ? push_launch<8, 1, EV, SP> : push_launch<4, 1, EV, SP>);
     };
-    if (g.order == 2) {
-        if (g.T == 8) launch(k_push_deposit<8, 2>, 2);
-        else launch(k_push_deposit<4, 2>, 3);
-    } else {
-        if (g.T == 8) launch(k_push_deposit<8, 1>, 0);
-        else launch(k_push_deposit<4, 1>, 1);
-    }
+    const std::true_type yes;
+    const std::false_type no;
+    if (events) split > 1 ? shape(yes, yes) : shape(yes, no);
+    else split > 1 ? shape(no, yes) : shape(no, no);
 }
 
 void launch_j_reduce(const GridDev &g, const float *jscratch, const int *jvalid, float *J, cudaStream_t st) {

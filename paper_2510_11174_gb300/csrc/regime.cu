@@ -53,17 +53,22 @@ __device__ __forceinline__ void tile_origin(const GridDev &g, int t, int o[3]) {
 
 // add v times the CIC weights of a particle at pos (unwrapped, inside the
 // frame) to component q of a fixed-point frame
-__device__ __forceinline__ void frame_cic(const GridDev &g, unsigned long long *fr, int G, const int o[3],
+__device__ __forceinline__ void frame_cic(const GridDev &g, unsigned *fr, int n, int G, const int o[3],
                                           const float pos[3], float v) {
     int b[3];
     float f[3];
     for (int a = 0; a < 3; ++a) cic_axis(g, a, pos[a], b[a], f[a]);
+    int idx[8];
+    float val[8];
+#pragma unroll
     for (int c = 0; c < 8; ++c) {
         const float wgt = ((c & 1) ? f[0] : 1.0f - f[0]) * (((c >> 1) & 1) ? f[1] : 1.0f - f[1]) *
                           ((c >> 2) ? f[2] : 1.0f - f[2]);
         const int l0 = b[0] + (c & 1) - o[0], l1 = b[1] + ((c >> 1) & 1) - o[1], l2 = b[2] + (c >> 2) - o[2];
-        if (wgt != 0.0f) atomicAdd(&fr[(l2 * G + l1) * G + l0], fix_of(wgt * v));
+        idx[c] = (l2 * G + l1) * G + l0;
+        val[c] = wgt != 0.0f ? wgt * v : 0.0f;
     }
+    fix_add<8>(fr, n, idx, val);
 }
 
 // a particle position of tile t is inside the tile's cells (what the frames assume)
@@ -85,7 +90,7 @@ __global__ void __launch_bounds__(256) k_density_frames(GridDev g, const SpDev *
                                                          unsigned which, int charge, float *__restrict__ scratch,
                                                          int *__restrict__ valid, int *__restrict__ status) {
     extern __shared__ __align__(16) unsigned char smraw[];
-    unsigned long long *fr = reinterpret_cast<unsigned long long *>(smraw);
+    unsigned *fr = reinterpret_cast<unsigned *>(smraw);
     __shared__ int s_max[32];
     const int t = blockIdx.x, G = frame_G(g.T), G3 = G * G * G;
     const float idV = 1.0f / (g.d[0] * g.d[1] * g.d[2]);
@@ -105,7 +110,7 @@ __global__ void __launch_bounds__(256) k_density_frames(GridDev g, const SpDev *
         return;
     }
     block_max_put(vmax, s_max);
-    for (int l = threadIdx.x; l < G3; l += blockDim.x) fr[l] = 0ULL;
+    for (int l = threadIdx.x; l < 2 * G3; l += blockDim.x) fr[l] = 0u;
     __syncthreads();
     const int k = fix_exponent((double)total * (double)block_max_read(s_max));
     const float sc = pow2f(k);
@@ -124,13 +129,13 @@ __global__ void __launch_bounds__(256) k_density_frames(GridDev g, const SpDev *
                 atomicOr(status, ST_BADPOS);
                 continue;
             }
-            frame_cic(g, fr, G, o, pos, qv * sp.w[base + p] * (zq ? zq[base + p] : 1.0f));
+            frame_cic(g, fr, G3, G, o, pos, qv * sp.w[base + p] * (zq ? zq[base + p] : 1.0f));
         }
     }
     __syncthreads();
     float *dst = scratch + (long long)t * G3;
     const float inv = pow2f(-k);
-    for (int l = threadIdx.x; l < G3; l += blockDim.x) dst[l] = fix_to_float(fr[l], inv);
+    for (int l = threadIdx.x; l < G3; l += blockDim.x) dst[l] = fix_to_float(fix_read(fr, G3, l), inv);
     if (threadIdx.x == 0) valid[t] = 1;
 }
 
@@ -286,7 +291,7 @@ __global__ void __launch_bounds__(256) k_fluid_to_particles(GridDev g, const uin
                                                              float *__restrict__ scratch, int *__restrict__ valid,
                                                              int *__restrict__ status) {
     extern __shared__ __align__(16) unsigned char smraw[];
-    unsigned long long *fr = reinterpret_cast<unsigned long long *>(smraw);
+    unsigned *fr = reinterpret_cast<unsigned *>(smraw);
     __shared__ int s_max[32];
     const int t = blockIdx.x, T = g.T, G = frame_G(T), G3 = G * G * G, T3 = T * T * T;
     int o[3];
@@ -316,7 +321,7 @@ __global__ void __launch_bounds__(256) k_fluid_to_particles(GridDev g, const uin
         return;
     }
     block_max_put(qmax, s_max);
-    for (int l = threadIdx.x; l < G3; l += blockDim.x) fr[l] = 0ULL;
+    for (int l = threadIdx.x; l < 2 * G3; l += blockDim.x) fr[l] = 0u;
     __syncthreads();
     // each converting node adds q n at itself and -q n spread by CIC: a node's
     // sum is at most 2 T^3 max |q n|
@@ -333,7 +338,9 @@ __global__ void __launch_bounds__(256) k_fluid_to_particles(GridDev g, const uin
         const float w = n * dV / (float)ppc;
         {
             const int l0 = idx[0] - o[0], l1 = idx[1] - o[1], l2 = idx[2] - o[2];
-            atomicAdd(&fr[(l2 * G + l1) * G + l0], fix_of(f.q * n * sc));
+            const int at[1] = {(l2 * G + l1) * G + l0};
+            const float val[1] = {f.q * n * sc};
+            fix_add<1>(fr, G3, at, val);
         }
         const float u[3] = {f.ux[c], f.uy[c], f.uz[c]};
         for (int p = 0; p < ppc; ++p) {
@@ -357,7 +364,7 @@ __global__ void __launch_bounds__(256) k_fluid_to_particles(GridDev g, const uin
             }
             // CIC charge of the new particle leaves rho_bg (the unwrapped
             // position indexes the frame; the gather wraps periodic axes)
-            frame_cic(g, fr, G, o, upos, -dst.q * w / dV * sc);
+            frame_cic(g, fr, G3, G, o, upos, -dst.q * w / dV * sc);
             const uint64_t id = (1ULL << 62) | (derived_id((uint64_t)c | ((uint64_t)epoch << 40), p, 6u) >> 2);
             const float tau = dst.tau ? tau_initial(id, g.seed, dst.tau_index) : 0.0f;
             tile_put(dst, tile_index(g, pos[0], pos[1], pos[2]), pos, u, w, id, tau, status);
@@ -368,7 +375,7 @@ __global__ void __launch_bounds__(256) k_fluid_to_particles(GridDev g, const uin
     __syncthreads();
     float *out = scratch + (long long)t * G3;
     const float inv = pow2f(-k);
-    for (int l = threadIdx.x; l < G3; l += blockDim.x) out[l] = fix_to_float(fr[l], inv);
+    for (int l = threadIdx.x; l < G3; l += blockDim.x) out[l] = fix_to_float(fix_read(fr, G3, l), inv);
     if (threadIdx.x == 0) valid[t] = 1;
 }
 
@@ -390,7 +397,7 @@ __global__ void __launch_bounds__(256) k_particles_to_fluid(GridDev g, const uin
                                                              float *__restrict__ scratch, int *__restrict__ valid,
                                                              int *__restrict__ status) {
     extern __shared__ __align__(16) unsigned char smraw[];
-    unsigned long long *fr = reinterpret_cast<unsigned long long *>(smraw);  // n, n ux, n uy, n uz
+    unsigned *fr = reinterpret_cast<unsigned *>(smraw);  // n, n ux, n uy, n uz
     __shared__ int s_holes;
     __shared__ int s_max[2][32];
     const int t = blockIdx.x, G = frame_G(g.T), G3 = G * G * G;
@@ -431,7 +438,7 @@ __global__ void __launch_bounds__(256) k_particles_to_fluid(GridDev g, const uin
     }
     block_max_put(wmax, s_max[0]);
     block_max_put(wumax, s_max[1]);
-    for (int l = threadIdx.x; l < 4 * G3; l += blockDim.x) fr[l] = 0ULL;
+    for (int l = threadIdx.x; l < 8 * G3; l += blockDim.x) fr[l] = 0u;
     __syncthreads();
     const int kn = fix_exponent((double)n * (double)block_max_read(s_max[0]));
     const int ku = fix_exponent((double)n * (double)block_max_read(s_max[1]));
@@ -445,10 +452,10 @@ __global__ void __launch_bounds__(256) k_particles_to_fluid(GridDev g, const uin
             continue;
         }
         const float wn = sp.w[s] * idV;
-        frame_cic(g, fr, G, o, pos, wn * sn);
-        frame_cic(g, fr + G3, G, o, pos, wn * sp.ux[s] * su);
-        frame_cic(g, fr + 2 * G3, G, o, pos, wn * sp.uy[s] * su);
-        frame_cic(g, fr + 3 * G3, G, o, pos, wn * sp.uz[s] * su);
+        frame_cic(g, fr, 4 * G3, G, o, pos, wn * sn);
+        frame_cic(g, fr + G3, 4 * G3, G, o, pos, wn * sp.ux[s] * su);
+        frame_cic(g, fr + 2 * G3, 4 * G3, G, o, pos, wn * sp.uy[s] * su);
+        frame_cic(g, fr + 3 * G3, 4 * G3, G, o, pos, wn * sp.uz[s] * su);
         const int h = atomicAdd(&s_holes, 1);
         sp.holes[base + h] = p;
         sp.x[s] = -1.0f;
@@ -456,7 +463,7 @@ __global__ void __launch_bounds__(256) k_particles_to_fluid(GridDev g, const uin
     __syncthreads();
     float *out = scratch + (long long)t * 4 * G3;
     const float in_ = pow2f(-kn), iu = pow2f(-ku);
-    for (int l = threadIdx.x; l < 4 * G3; l += blockDim.x) out[l] = fix_to_float(fr[l], l < G3 ? in_ : iu);
+    for (int l = threadIdx.x; l < 4 * G3; l += blockDim.x) out[l] = fix_to_float(fix_read(fr, 4 * G3, l), l < G3 ? in_ : iu);
     if (threadIdx.x == 0) {
         valid[t] = 1;
         sp.hole_count[t] = s_holes;
