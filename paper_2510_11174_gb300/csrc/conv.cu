@@ -7,37 +7,42 @@
 // and warp-specialised.  The three x-taps of the stencil go into the N
 // dimension: for each of the 9 (dz, dy) taps one tcgen05.mma multiplies the
 // 128 input cells of a 16 (x) x 8 (y) x 1 (z) block, shifted by (dz, dy), by
-// the weights of all three x-taps side by side (N = 3 C_out), so every A tile
-// read from shared memory feeds three times the math (the A-operand fetch,
-// not the math, limits narrow layers).  The epilogue adds the three partial
-// sums of neighbouring x cells (lanes m - 1, m, m + 1, one warp shuffle each
-// way), so a tile yields the 14 (x) x 8 (y) interior outputs of its block;
-// tiles step by 14 cells in x.  The block halo (16 x 10 x 3 cells) is
-// fetched by TMA, one 16-channel block per copy, into a ring of 5 to 8
-// shared-memory buffers laid out [block][z][y][x][16 channels] with the
-// 32-byte swizzle (the TMA and the tensor core both apply it to the absolute
-// shared address, so an operand may start at any cell of the halo); all
-// 27 x C_in x C_out weights stay resident in shared memory.
-//   warp 0      TMA producer: waits for a free stage, posts the expected bytes
-//               on the stage's "full" barrier and issues the chunk copies
-//               (zero fill outside the volume comes from the tensor map);
-//   warp 1      MMA issuer: per tile 9 taps x C_in/16 tcgen05.mma of shape
-//               M = 128 cells x N = 3 C_out x K = 16 into one of 2 or 4 TMEM
-//               accumulators; commits free the stage and hand the
-//               accumulator to the epilogue;
-//   warps 2..   epilogue, one warp per TMEM lane quarter and 8-channel
-//               output group (4 C_out / 8 warps; warp w reads TMEM lanes
-//               32 (w % 4) .. and channels 8 ((w - 2) / 4) ..): tcgen05.ld of
-//               the accumulator rows, the x-tap sum across lanes, bias, ReLU,
-//               Philox dropout with inverted scaling, channels-last stores.
-//               What does not depend on the accumulator (the tile position,
-//               stepped with carries; the cell's validity; the dropout bits;
-//               the bias) is computed before waiting for it, so it overlaps
-//               the MMAs instead of lengthening the epilogue's chain.
-// The operand of tap (dz, dy) is the halo shifted by that tap: its 128 cells
-// are 128 consecutive 32-byte rows (one swizzle atom wide in K, 8-row groups
-// 256 bytes apart), so every tap and 16-channel block is a plain K-major SW32
-// matrix descriptor -- no im2col.
+// the weights of all three x-taps side by side (3 C_out columns), so every A
+// tile read from shared memory feeds three times the math.  The epilogue adds
+// the three partial sums of neighbouring x cells (lanes m - 1, m, m + 1, one
+// warp shuffle each way), so a block yields its 14 (x) x 8 (y) interior
+// outputs; blocks step by 14 cells in x.
+// A CTA walks a column of blocks along z: each plane of the halo (16 x 10
+// cells, all channels) is fetched once by TMA into a ring of planes and used by
+// the three output planes it touches.  With 16 outputs the three z-taps go into
+// N too (ZN = 3): one MMA of 144 columns adds a plane's share to the
+// accumulators of three output planes at once, which lie side by side in a ring
+// of TMEM slots.  In every layout an output's sum is formed in the same order
+// (per x-tap: dz, dy, 16-channel block; then left + middle + right).
+//   warp 0      TMA producer: waits for a free plane, posts the expected bytes
+//               on its "full" barrier and issues the copy (zero fill outside
+//               the volume comes from the tensor map);
+//   warp 1      MMA issuer (M = 128 cells x K = 16 per instruction) into a ring
+//               of 5 (32 outputs) or 10 (16 outputs) TMEM accumulators; commits
+//               free the plane and hand the accumulator to the epilogue;
+//   warps 2..17 epilogue, one warp per TMEM lane quarter and 16-channel output
+//               group, in 2 (32 outputs) or 4 (16 outputs) sets that take the
+//               output planes in turn: tcgen05.ld of the accumulator rows, the
+//               x-tap sum across lanes, bias, ReLU, Philox dropout with inverted
+//               scaling, channels-last stores.  What does not depend on the
+//               accumulator (dropout bits, bias) is computed before waiting for
+//               it.
+// What bounds it: an MMA takes max(N / 2, (4 KB + 32 N B) / 128 B) cycles (the
+// math, or fetching its operands from shared memory: 56 at N = 96, 44 at N =
+// 48, 72 at N = 144, measured in a chain of 1800), and the TMA's writes take
+// about a cycle per cell and 64 B on the same shared-memory port.  Walking along
+// z with 64-byte rows writes 160 cells per output plane; a halo of three planes
+// per block in 32-byte rows wrote 960, as much as the MMAs' own 1008 cycles.
+// The operand of tap (dz, dy) is a plane shifted by dy rows: its 128 cells are
+// 128 consecutive rows of 64 (32 input channels) or 32 bytes (16), so every tap
+// and 16-channel block is a plain K-major swizzled matrix descriptor -- no
+// im2col; the TMA and the tensor core both apply the swizzle to the absolute
+// shared address, so an operand may start at any row.
 // Every wait is bounded: a wait that gives up sets ST_TIMEOUT, the roles stop
 // issuing work, copies and MMAs in flight are waited for (bounded) and TMEM
 // is released.
@@ -54,10 +59,9 @@ namespace hyb {
 
 static constexpr int TX = 16, TY = 8;                 // A block (cells): M = 128 rows
 static constexpr int TXO = TX - 2;                     // output cells per block row (the interior)
-static constexpr int HY = TY + 2, HZ = 3;              // halo (x needs none: the x-taps live in N)
-static constexpr int HCELLS = TX * HY * HZ;            // 480
-static constexpr int CHB = HCELLS * 32;                // bytes one 16-channel copy writes (15360)
-static constexpr int CHBP = (CHB + 1023) / 1024 * 1024; // block pitch in shared memory (15360)
+static constexpr int HY = TY + 2;                      // halo rows of a plane (x needs none: the x-taps live in N)
+static constexpr int PCELLS = TX * HY;                 // cells of a plane (160)
+static constexpr int EPC = 16;                         // output channels per epilogue warp
 static constexpr long long MBAR_LIMIT = 1LL << 26;     // polls before a wait gives up
 
 // dropout keep decision of channel ch at cell (b, lin): Philox counter
@@ -86,286 +90,382 @@ __host__ __device__ inline void conv_tiles_x(int W, int x_lo, int x_hi, int &tx0
     }
 }
 
-// position of a persistent CTA's tile in (x tile, y tile, z, batch) digits,
-// stepped by the grid size with carries instead of divisions
-struct TileCursor {
-    int tx, ty, z, b;        // the current tile
-    int sx, sy, sz, sb;      // the step (grid size) in the same digits
-    int nx, ny, nz;
-    __device__ void init(uint32_t t, uint32_t step, int nx_, int ny_, int nz_) {
-        nx = nx_;
-        ny = ny_;
-        nz = nz_;
-        tx = (int)(t % (uint32_t)nx);
-        t /= (uint32_t)nx;
-        ty = (int)(t % (uint32_t)ny);
-        t /= (uint32_t)ny;
-        z = (int)(t % (uint32_t)nz);
-        b = (int)(t / (uint32_t)nz);
-        sx = (int)(step % (uint32_t)nx);
-        step /= (uint32_t)nx;
-        sy = (int)(step % (uint32_t)ny);
-        step /= (uint32_t)ny;
-        sz = (int)(step % (uint32_t)nz);
-        sb = (int)(step / (uint32_t)nz);
-    }
-    __device__ void next() {
-        tx += sx;
-        int c = tx >= nx;
-        tx -= c ? nx : 0;
-        ty += sy + c;
-        c = ty >= ny;
-        ty -= c ? ny : 0;
-        z += sz + c;
-        c = z >= nz;
-        z -= c ? nz : 0;
-        b += sb + c;
+// a column of blocks: x tile, y tile, output planes z0 .. z1 - 1, batch
+struct ConvUnit {
+    int tx, ty, z0, z1, b;
+};
+__device__ __forceinline__ ConvUnit conv_unit(long long u, int tx0, int nx, int ny, int nzc, int lz, int D) {
+    ConvUnit c;
+    uint32_t t = (uint32_t)u;  // unit counts fit in 32 bits (checked at launch)
+    c.tx = (int)(t % (uint32_t)nx) + tx0;
+    t /= (uint32_t)nx;
+    c.ty = (int)(t % (uint32_t)ny);
+    t /= (uint32_t)ny;
+    c.z0 = (int)(t % (uint32_t)nzc) * lz;
+    c.b = (int)(t / (uint32_t)nzc);
+    c.z1 = min(c.z0 + lz, D);
+    return c;
+}
+
+// index of a ring of S entries and the parity of its current round
+template <int S>
+struct Ring {
+    int s = 0;
+    uint32_t ph = 0;
+    __device__ __forceinline__ void next() {
+        if (++s == S) {
+            s = 0;
+            ph ^= 1;
+        }
     }
 };
 
 template <int KC, int N>
 struct ConvCfg {
-    static constexpr int NP = 3 * N;                   // MMA N: the three x-taps side by side
-    static constexpr int WBYTES = 27 * KC * N * 16;    // weights, core layout [9][KC][3 N][8]
-    static constexpr int RING = (WBYTES + 1023) / 1024 * 1024;  // halo ring offset (swizzle-aligned)
-    static constexpr int STAGE = (KC / 2) * CHBP;      // one halo buffer (16-channel blocks)
-    // as many halo buffers as shared memory holds (up to 8): the copies in
-    // flight must cover the L2 latency of a stage
-    static constexpr int SMEM_MAX = 227 * 1024 - 512;  // dynamic share (static barriers take the rest)
-    static constexpr int STAGES = (SMEM_MAX - 1024 - RING) / STAGE > 8 ? 8 : (SMEM_MAX - 1024 - RING) / STAGE;
-    static constexpr int SMEM = RING + STAGES * STAGE + 1024;  // + alignment slack
-    // TMEM accumulators: four when they fit the 512 columns (the MMAs may run
-    // three tiles ahead of the slowest epilogue warp), else two
-    static constexpr int NACC = 4 * NP <= 512 ? 4 : 2;
-    static constexpr int TCOLS = NACC * NP <= 32 ? 32 : (NACC * NP <= 64 ? 64 : (NACC * NP <= 128 ? 128 :
-                                 (NACC * NP <= 256 ? 256 : 512)));
-    static constexpr int NG = N / 8;                   // 8-channel output groups
-    static constexpr int NEPI = 4 * NG;                // epilogue warps: one per lane quarter and group
-    static constexpr int NTHREADS = 64 + 32 * NEPI;    // + producer and MMA issuer
+    static constexpr int NP = 3 * N;                   // columns of one accumulator: the three x-taps side by side
+    static constexpr int ZN = N == 16 ? 3 : 1;         // output planes one MMA adds to
+    static constexpr int ROWB = KC * 16;               // bytes of a cell in shared memory
+    static constexpr int WBYTES = 27 * KC * N * 16;    // weights, core layout [9 (dz, dy) or 3 (dy)][KC][ZN 3 N][8]
+    static constexpr int RING = (WBYTES + 1023) / 1024 * 1024;  // plane ring offset (swizzle-aligned)
+    static constexpr int PLANE = PCELLS * ROWB;        // a multiple of 1024
+    static constexpr int SMEM_MAX = 227 * 1024 - 1024; // dynamic share (static barriers take the rest)
+    static constexpr int FIT = (SMEM_MAX - 1024 - RING) / PLANE;
+    static constexpr int PLANES = FIT > 16 ? 16 : FIT; // the copies in flight must cover the L2 latency of a plane
+    static constexpr int SMEM = RING + PLANES * PLANE + 1024;  // + alignment slack
+    static constexpr int NACC = 480 / NP;              // TMEM accumulators
+    static constexpr int NG = N / EPC;                 // 16-channel output groups
+    static constexpr int NSET = 4 / NG;                // epilogue sets (16 warps in all)
+    static constexpr int NTHREADS = 64 + 512;          // producer, MMA issuer, epilogue
 };
 
 template <int KC, int N>
 __global__ void __launch_bounds__(ConvCfg<KC, N>::NTHREADS, 1)
     k_conv3_tc(const __grid_constant__ CUtensorMap tmap, ConvArgs a) {
     using Cfg = ConvCfg<KC, N>;
+    constexpr int PLANES = Cfg::PLANES, NACC = Cfg::NACC, NP = Cfg::NP, ZN = Cfg::ZN;
+    static_assert(PLANES >= 5 && Cfg::PLANE % 1024 == 0, "plane ring");
     extern __shared__ uint8_t smem_raw[];
-    // 1024-byte aligned base: weights first, then the halo ring
+    // 1024-byte aligned base: weights first, then the plane ring
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t *wsm = smem;
     uint8_t *ring = smem + Cfg::RING;
-    constexpr int STAGES = Cfg::STAGES;
-    static_assert(STAGES >= 2, "shared memory holds fewer than two halo buffers");
-    __shared__ __align__(8) uint64_t full_b[STAGES], empty_b[STAGES], tfull_b[Cfg::NACC], tempty_b[Cfg::NACC], done_b;
+    __shared__ __align__(8) uint64_t full_b[PLANES], empty_b[PLANES], tfull_b[NACC], tempty_b[NACC], wfull_b, done_b;
     __shared__ uint32_t taddr_s;
     __shared__ int abort_s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     if (warp == 1) {
-        tmem_alloc(smem_u32(&taddr_s), Cfg::TCOLS);
+        tmem_alloc(smem_u32(&taddr_s), 512);
         tmem_relinquish();
     }
     if (tid == 0) {
-        for (int s = 0; s < STAGES; ++s) {
+        for (int s = 0; s < PLANES; ++s) {
             mbar_init(smem_u32(&full_b[s]), 1);
             mbar_init(smem_u32(&empty_b[s]), 1);
         }
-        for (int k = 0; k < Cfg::NACC; ++k) {
+        for (int k = 0; k < NACC; ++k) {
             mbar_init(smem_u32(&tfull_b[k]), 1);
-            mbar_init(smem_u32(&tempty_b[k]), Cfg::NEPI);
+            mbar_init(smem_u32(&tempty_b[k]), 4 * Cfg::NG);
         }
+        mbar_init(smem_u32(&wfull_b), 1);
         mbar_init(smem_u32(&done_b), 1);
         abort_s = 0;
         fence_mbar_init();
         prefetch_tmap(&tmap);
+        // weights by bulk copies while TMEM is allocated and the first planes arrive; they
+        // are in core layout [9 (dz, dy)][KC][NP] already, with ZN = 3 the rows of the
+        // three dz of one dy go side by side, dz = 2 (the plane below) first
+        const uint32_t wb = smem_u32(&wfull_b), w0 = smem_u32(wsm);
+        mbar_arrive_expect_tx(wb, Cfg::WBYTES);
+        if (ZN == 1) {
+            bulk_load(w0, a.wt, Cfg::WBYTES, wb);
+        } else {
+            const char *src = reinterpret_cast<const char *>(a.wt);
+            for (int i = 0; i < 9 * KC; ++i) {
+                const int z = i % 3, kc = (i / 3) % KC, dy = i / (3 * KC);
+                bulk_load(w0 + (uint32_t)(i * NP * 16), src + (((2 - z) * 3 + dy) * KC + kc) * NP * 16, NP * 16, wb);
+            }
+        }
     }
-    // weights: straight 16-byte copies (already in core layout)
-    {
-        const uint4 *src = reinterpret_cast<const uint4 *>(a.wt);
-        uint4 *dst = reinterpret_cast<uint4 *>(wsm);
-        for (int i = tid; i < Cfg::WBYTES / 16; i += Cfg::NTHREADS) dst[i] = src[i];
-    }
-    fence_proxy_async_smem();
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
     const uint32_t taddr = taddr_s;
     int tx0, tiles_x;
     conv_tiles_x(a.W, a.x_lo, a.x_hi, tx0, tiles_x);
-    const int tiles_y = a.H / TY;
-    const long long ntiles = (long long)a.B * a.D * tiles_y * tiles_x;
+    const int tiles_y = a.H / TY, nzc = (a.D + a.lz - 1) / a.lz;
+    const long long nunits = (long long)a.B * nzc * tiles_y * tiles_x;
     const uint32_t ring_s = smem_u32(ring), w_s = smem_u32(wsm);
 
     if (warp == 0) {
         // ------------------------------------------------------------ producer
         if (lane == 0) {
-            int s = 0;
-            uint32_t ph = 0;
+            Ring<PLANES> r;
             long long issued = 0;
-            TileCursor cur;
-            cur.init(blockIdx.x, gridDim.x, tiles_x, tiles_y, a.D);
-            for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x, cur.next()) {
-                if (!mbar_wait(smem_u32(&empty_b[s]), ph ^ 1, MBAR_LIMIT) || *(volatile int *)&abort_s) {
-                    atomicOr(a.status, ST_TIMEOUT);
-                    *(volatile int *)&abort_s = 1;
-                    break;
-                }
-                const int tx = cur.tx + tx0, ty = cur.ty, z0 = cur.z, b = cur.b;
-                const uint32_t fb = smem_u32(&full_b[s]);
-                mbar_arrive_expect_tx(fb, (KC / 2) * CHB);
-                const uint32_t dst = ring_s + (uint32_t)(s * Cfg::STAGE);
-#pragma unroll
-                for (int c = 0; c < KC / 2; ++c)
-                    tma_load_5d(dst + (uint32_t)(c * CHBP), &tmap, a.cin_off + 16 * c, tx * TXO - 1, ty * TY - 1, z0 - 1,
-                                b, fb);
-                ++issued;
-                if (++s == STAGES) {
-                    s = 0;
-                    ph ^= 1;
+            bool stop = false;
+            for (long long u = blockIdx.x; u < nunits && !stop; u += gridDim.x) {
+                const ConvUnit c = conv_unit(u, tx0, tiles_x, tiles_y, nzc, a.lz, a.D);
+                for (int p = c.z0 - 1; p <= c.z1; ++p) {
+                    if (!mbar_wait_abort(smem_u32(&empty_b[r.s]), r.ph ^ 1, MBAR_LIMIT, &abort_s)) {
+                        atomicOr(a.status, ST_TIMEOUT);
+                        *(volatile int *)&abort_s = 1;
+                        stop = true;
+                        break;
+                    }
+                    const uint32_t fb = smem_u32(&full_b[r.s]);
+                    mbar_arrive_expect_tx(fb, Cfg::PLANE);
+                    tma_load_5d(ring_s + (uint32_t)(r.s * Cfg::PLANE), &tmap, a.cin_off, c.tx * TXO - 1, c.ty * TY - 1,
+                                p, c.b, fb);
+                    ++issued;
+                    r.next();
                 }
             }
             // copies still in flight when the loop stopped early complete before exit
             if (*(volatile int *)&abort_s) {
-                for (int k = 0; k < STAGES && issued > 0; ++k, --issued) {
-                    if (--s < 0) {
-                        s = STAGES - 1;
-                        ph ^= 1;
+                for (int k = 0; k < PLANES && issued > 0; ++k, --issued) {
+                    if (--r.s < 0) {
+                        r.s = PLANES - 1;
+                        r.ph ^= 1;
                     }
-                    mbar_wait(smem_u32(&full_b[s]), ph, MBAR_LIMIT);
+                    mbar_wait(smem_u32(&full_b[r.s]), r.ph, MBAR_LIMIT);
                 }
             }
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            constexpr uint32_t idesc = idesc_bf16(128, Cfg::NP);
-            const uint64_t a0 = smem_desc_sw32(ring_s, 8 * 32);
-            const uint64_t b0 = smem_desc(w_s, Cfg::NP * 16, 128);
-            int s = 0;
-            uint32_t ph = 0;
-            long long it = 0;
-            for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
-                const int acc = (int)(it % Cfg::NACC);
-                const uint32_t aph = (uint32_t)((it / Cfg::NACC) & 1);
-                if (!mbar_wait(smem_u32(&tempty_b[acc]), aph ^ 1, MBAR_LIMIT) ||
-                    !mbar_wait(smem_u32(&full_b[s]), ph, MBAR_LIMIT) || *(volatile int *)&abort_s) {
-                    atomicOr(a.status, ST_TIMEOUT);
-                    *(volatile int *)&abort_s = 1;
+        // (the whole warp runs the loop; an elected lane issues)
+        const uint64_t a0 = KC == 4 ? smem_desc_sw64(0, 8 * 64) : smem_desc_sw32(0, 8 * 32);
+        const uint64_t b0 = smem_desc(0, ZN * NP * 16, 128);
+        const uint32_t ahi = (uint32_t)(a0 >> 32), bhi = (uint32_t)(b0 >> 32);
+        const uint32_t alo = (uint32_t)a0 + (ring_s >> 4), blo = (uint32_t)b0 + (w_s >> 4);  // below 2^14: no carry
+        Ring<PLANES> pr;       // the plane being waited for
+        Ring<NACC> ar;         // the accumulator of the next output plane to begin
+        LookAhead<PLANES, NACC> look;
+        if (!mbar_wait_abort(smem_u32(&wfull_b), 0, MBAR_LIMIT, &abort_s) && lane == 0) {
+            atomicOr(a.status, ST_TIMEOUT);
+            *(volatile int *)&abort_s = 1;
+        }
+        int ps[3] = {0, 0, 0}; // ring slots of planes p - 2, p - 1, p
+        bool stop = false;
+        for (long long u = blockIdx.x; u < nunits && !stop; u += gridDim.x) {
+            const ConvUnit c = conv_unit(u, tx0, tiles_x, tiles_y, nzc, a.lz, a.D);
+            int s0 = ar.s;     // accumulator of output plane max(p - 1, z0)
+            for (int p = c.z0 - 1; p <= c.z1; ++p) {
+                ps[0] = ps[1];
+                ps[1] = ps[2];
+                ps[2] = pr.s;
+                // the output plane that this plane begins
+                const bool begins = ZN == 3 ? p + 1 < c.z1 : p - 1 >= c.z0;
+                if (!look.wait(full_b, pr.s, pr.ph, tempty_b, ar.s, ar.ph ^ 1, begins, lane, MBAR_LIMIT, &abort_s)) {
+                    if (lane == 0) {
+                        atomicOr(a.status, ST_TIMEOUT);
+                        *(volatile int *)&abort_s = 1;
+                    }
+                    stop = true;
+                    break;
+                }
+                pr.next();
+                fence_after_sync();
+                if constexpr (ZN == 1) {
+                    if (p - 1 < c.z0) continue;
+                    const uint32_t d = taddr + (uint32_t)(ar.s * NP);
+                    constexpr uint32_t idesc = idesc_bf16(128, NP);
+#pragma unroll
+                    for (int dz = 0; dz < 3; ++dz) {
+                        const uint32_t ad = alo + (uint32_t)((ps[dz] * Cfg::PLANE) >> 4);
+#pragma unroll
+                        for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+                            for (int kk = 0; kk < KC / 2; ++kk)
+                                umma_bf16_warp(d, ad + (uint32_t)((dy * TX * Cfg::ROWB + kk * 32) >> 4), ahi,
+                                               blo + (uint32_t)((((dz * 3 + dy) * KC + 2 * kk) * NP * 16) >> 4), bhi, idesc,
+                                               (dz | dy | kk) != 0);
+                    }
+                    umma_commit_warp(smem_u32(&empty_b[ps[0]]));   // the lowest plane may be refilled
+                    if (p == c.z1) {
+                        umma_commit_warp(smem_u32(&empty_b[ps[1]]));
+                        umma_commit_warp(smem_u32(&empty_b[ps[2]]));
+                    }
+                    umma_commit_warp(smem_u32(&tfull_b[ar.s]));    // the accumulator is ready
+                    ar.next();
+                } else {
+                    const uint32_t ad = alo + (uint32_t)(ps[2] * (Cfg::PLANE >> 4));
+                    if (p > c.z0 && begins && s0 + 2 < NACC) {
+                        // inside a column: three output planes in accumulators s0 .. s0 + 2, the
+                        // last one begun (its first product overwrites it); constants only
+                        const uint32_t d = taddr + (uint32_t)(s0 * NP);
+                        umma_bf16_warp(d, ad, ahi, blo, bhi, idesc_bf16(128, 2 * NP), 1);
+                        umma_bf16_warp(d + 2 * NP, ad, ahi, blo + 2 * NP, bhi, idesc_bf16(128, NP), 0);
+#pragma unroll
+                        for (int i = 1; i < 3 * KC / 2; ++i)
+                            umma_bf16_warp(d, ad + (uint32_t)(((i / (KC / 2)) * TX * Cfg::ROWB + (i % (KC / 2)) * 32) >> 4),
+                                           ahi, blo + (uint32_t)(i * 6 * NP), bhi, idesc_bf16(128, 3 * NP), 1);
+                    } else {
+                        // output planes lo .. hi (dz = p - z + 1), in consecutive accumulators from s0
+                        const int lo = max(p - 1, c.z0), hi = min(p + 1, c.z1 - 1), n = hi - lo + 1;
+                        const uint32_t bd = blo + (uint32_t)(((lo - p + 1) * NP * 16) >> 4);
+                        auto mma = [&](int dy, int kk, int first, int cnt, uint32_t acc) {
+                            const int sl = s0 + first;
+                            umma_bf16_warp(taddr + (uint32_t)((sl < NACC ? sl : sl - NACC) * NP),
+                                           ad + (uint32_t)((dy * TX * Cfg::ROWB + kk * 32) >> 4), ahi,
+                                           bd + (uint32_t)(first * NP) + (uint32_t)(((dy * KC + 2 * kk) * 3 * NP * 16) >> 4),
+                                           bhi, idesc_bf16(128, 8) - (1u << 17) + ((uint32_t)(cnt * NP) << 14), acc);
+                        };
+                        // the first product of a new accumulator overwrites it
+                        const int old = begins ? n - 1 : n, n1 = min(n, NACC - s0), o1 = min(old, n1);
+                        if (o1 > 0) mma(0, 0, 0, o1, 1);
+                        if (old > o1) mma(0, 0, o1, old - o1, 1);
+                        if (begins) mma(0, 0, n - 1, 1, 0);
+                        if (n1 == n) {
+#pragma unroll
+                            for (int i = 1; i < 3 * KC / 2; ++i) mma(i / (KC / 2), i % (KC / 2), 0, n, 1);
+                        } else {
+                            // the accumulator ring wraps
+#pragma unroll
+                            for (int i = 1; i < 3 * KC / 2; ++i) {
+                                mma(i / (KC / 2), i % (KC / 2), 0, n1, 1);
+                                mma(i / (KC / 2), i % (KC / 2), n1, n - n1, 1);
+                            }
+                        }
+                    }
+                    umma_commit_warp(smem_u32(&empty_b[ps[2]]));
+                    if (begins) ar.next();
+                    if (p - 1 >= c.z0) {
+                        umma_commit_warp(smem_u32(&tfull_b[s0]));  // output plane p - 1 is complete
+                        if (++s0 == NACC) s0 = 0;
+                    }
+                }
+            }
+        }
+        // every MMA issued has finished reading shared memory before exit
+        umma_commit_warp(smem_u32(&done_b));
+        mbar_wait(smem_u32(&done_b), 0, MBAR_LIMIT);
+    } else {
+        // ------------------------------------------------------------ epilogue
+        const int q = warp & 3;                    // TMEM lane quarter this warp may access
+        const int grp = ((warp - 2) >> 2) % Cfg::NG;  // its 16 output channels
+        const int set = ((warp - 2) >> 2) / Cfg::NG;  // its share of the output planes
+        const int m = q * 32 + lane;               // accumulator row = cell of the block
+        const float scale = a.scale_out ? a.drop_scale : 1.0f;
+        const uint64_t scale2 = f32x2(scale, scale);
+        const int bx = m & (TX - 1);               // cell of the block row (0 and TX - 1 are halo)
+        const long long opitch = a.out_pitch ? a.out_pitch : N;
+        const long long HW = (long long)a.H * a.W;
+        // dropout threshold in both halves; its top bits pick the compare below
+        const uint32_t thr = a.drop_thr, thr7 = (thr & 0x7FFFu) * 0x10001u, thr_low = thr < 0x8000u ? 0xFFFFFFFFu : 0u;
+        uint64_t bias[EPC / 2];
+#pragma unroll
+        for (int j = 0; j < EPC / 2; ++j)
+            bias[j] = a.bias ? f32x2(__ldg(a.bias + grp * EPC + 2 * j), __ldg(a.bias + grp * EPC + 2 * j + 1)) : 0ULL;
+        Ring<NACC> ar;
+        int turn = 0;
+        bool stop = false;
+        for (long long u = blockIdx.x; u < nunits && !stop; u += gridDim.x) {
+            const ConvUnit c = conv_unit(u, tx0, tiles_x, tiles_y, nzc, a.lz, a.D);
+            const int cx = c.tx * TXO + bx - 1, cy = c.ty * TY + (m >> 4);
+            // the halo cells of the block row, and cells past the volume, write nothing
+            const bool valid = bx != 0 && bx != TX - 1 && cx < a.W;
+            uint32_t lin = (uint32_t)(((long long)c.z0 * a.H + cy) * a.W + (valid ? cx : 0));
+            long long obase = ((((long long)c.b * a.D + c.z0) * a.H + cy) * a.W + (valid ? cx : 0)) * opitch +
+                              a.out_off + grp * EPC;
+            for (int z = c.z0; z < c.z1; ++z, lin += (uint32_t)HW, obase += HW * opitch, ar.next()) {
+                const bool mine = turn == set;
+                if (++turn == Cfg::NSET) turn = 0;
+                if (!mine) continue;
+                // first what does not need the accumulator (it overlaps the MMAs): the
+                // dropout masks, one half-word per channel (kept where its field >= threshold)
+                uint32_t keep[EPC / 2];
+#pragma unroll
+                for (int w = 0; w < EPC / 2; ++w) keep[w] = 0xFFFFFFFFu;
+                if (thr) {
+#pragma unroll
+                    for (int h = 0; h < EPC / 8; ++h) {
+                        const u32x4 r = philox4x32_10(lin, (uint32_t)c.b, (a.layer << 16) | (uint32_t)(grp * (EPC / 8) + h),
+                                                      a.pass, a.seed, 0xD0u);
+#pragma unroll
+                        for (int w = 0; w < 4; ++w) {
+                            // per half: bit 15 of t is (low 15 bits >= the threshold's)
+                            const uint32_t t = (r.v[w] | 0x80008000u) - thr7;
+                            const uint32_t ge = (r.v[w] & t) | (thr_low & (r.v[w] | t));
+                            asm("prmt.b32 %0, %1, 0, 0xBB99;" : "=r"(keep[h * 4 + w]) : "r"(ge));
+                        }
+                    }
+                }
+                const bool ok = mbar_wait_abort(smem_u32(&tfull_b[ar.s]), ar.ph, MBAR_LIMIT, &abort_s);
+                if (!__all_sync(0xffffffffu, ok)) {
+                    if (lane == 0) {
+                        atomicOr(a.status, ST_TIMEOUT);
+                        *(volatile int *)&abort_s = 1;
+                    }
+                    stop = true;
                     break;
                 }
                 fence_after_sync();
-                const uint32_t d = taddr + (uint32_t)(acc * Cfg::NP);
-                const uint64_t as = a0 + (uint64_t)((s * Cfg::STAGE) >> 4);
+                // row m holds, per x-tap dx, the partial sum of the outputs at cell
+                // x - dx + 1; the output at x is D_0[x - 1] + D_1[x] + D_2[x + 1]
+                uint64_t v2[EPC / 2];
+                {
+                    float p[3 * EPC];
+                    const uint32_t rowa = taddr + ((uint32_t)(q * 32) << 16) + (uint32_t)(ar.s * NP + grp * EPC);
+                    tmem_ld16x3(rowa, rowa + (uint32_t)N, rowa + (uint32_t)(2 * N), p);
+                    fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&tempty_b[ar.s]));
+                    // lanes m - 1 and m + 1 are the x-neighbours (same block row for
+                    // the interior cells that produce output)
 #pragma unroll
-                for (int tap = 0; tap < 9; ++tap) {
-                    const int dz = tap / 3, dy = tap % 3;
-                    const uint32_t toff = (uint32_t)((dz * HY + dy) * TX * 32);
-#pragma unroll
-                    for (int kk = 0; kk < KC / 2; ++kk) {
-                        const uint64_t ad = as + (uint64_t)((toff + (uint32_t)(kk * CHBP)) >> 4);
-                        const uint64_t bd = b0 + (uint64_t)(((tap * KC + 2 * kk) * Cfg::NP * 16) >> 4);
-                        umma_bf16(d, ad, bd, idesc, (tap | kk) != 0);
+                    for (int o = 0; o < EPC; o += 2) {
+                        const uint64_t left = f32x2(__shfl_up_sync(0xffffffffu, p[o], 1),
+                                                    __shfl_up_sync(0xffffffffu, p[o + 1], 1));
+                        const uint64_t right = f32x2(__shfl_down_sync(0xffffffffu, p[2 * EPC + o], 1),
+                                                     __shfl_down_sync(0xffffffffu, p[2 * EPC + o + 1], 1));
+                        v2[o / 2] = add2(add2(left, f32x2(p[EPC + o], p[EPC + o + 1])), right);
                     }
                 }
-                umma_commit(smem_u32(&empty_b[s]));    // the stage may be refilled
-                umma_commit(smem_u32(&tfull_b[acc]));  // the accumulator is ready
-                if (++s == STAGES) {
-                    s = 0;
-                    ph ^= 1;
-                }
-            }
-            // every MMA issued has finished reading shared memory before exit
-            umma_commit(smem_u32(&done_b));
-            mbar_wait(smem_u32(&done_b), 0, MBAR_LIMIT);
-        }
-    } else {
-        // ------------------------------------------------------------ epilogue
-        const int q = warp & 3;              // TMEM lane quarter this warp may access
-        const int grp = (warp - 2) >> 2;     // the 8 output channels 8 grp .. 8 grp + 7 of this warp
-        const int m = q * 32 + lane;         // accumulator row = cell of the tile
-        const float scale = a.drop_scale;
-        const int bx = m & (TX - 1);         // cell of the block row (0 and TX - 1 are halo)
-        const long long opitch = a.out_pitch ? a.out_pitch : N;
-        float bias8[8];
+                if (!valid) continue;
+                float v[EPC];
+                if (a.y_f32 && a.accum) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) bias8[j] = a.bias ? __ldg(a.bias + grp * 8 + j) : 0.0f;
-        TileCursor cur;                      // tile counts fit in 32 bits (checked at launch)
-        cur.init(blockIdx.x, gridDim.x, tiles_x, tiles_y, a.D);
-        long long it = 0;
-        for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it, cur.next()) {
-            // first what does not need the accumulator (it overlaps the MMAs):
-            // the cell, its validity and its dropout bits
-            const int tx = cur.tx + tx0, ty = cur.ty, z0 = cur.z, b = cur.b;
-            const int cx = tx * TXO + bx - 1, cy = ty * TY + (m >> 4);
-            // the halo cells of the block row, and cells past the volume, write nothing
-            const bool valid = bx != 0 && bx != TX - 1 && cx < a.W;
-            const uint32_t lin = (uint32_t)(((long long)z0 * a.H + cy) * a.W + (valid ? cx : 0));
-            const long long obase = ((((long long)b * a.D + z0) * a.H + cy) * a.W + (valid ? cx : 0)) * opitch +
-                                    a.out_off + grp * 8;
-            uint32_t keep16[4] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu};
-            if (a.drop_thr) {
-                const u32x4 r = philox4x32_10(lin, (uint32_t)b, (a.layer << 16) | (uint32_t)grp, a.pass, a.seed, 0xD0u);
-#pragma unroll
-                for (int w = 0; w < 4; ++w) keep16[w] = r.v[w];
-            }
-
-            const int acc = (int)(it % Cfg::NACC);
-            const uint32_t aph = (uint32_t)((it / Cfg::NACC) & 1);
-            const bool ok = mbar_wait(smem_u32(&tfull_b[acc]), aph, MBAR_LIMIT);
-            if (!__all_sync(0xffffffffu, ok) || *(volatile int *)&abort_s) {
-                if (lane == 0) {
-                    atomicOr(a.status, ST_TIMEOUT);
-                    *(volatile int *)&abort_s = 1;
-                }
-                break;
-            }
-            fence_after_sync();
-            // row m holds, per x-tap dx, the partial sum of the outputs at cell
-            // x - dx + 1; the output at x is D_0[x - 1] + D_1[x] + D_2[x + 1]
-            float v[8];
-            {
-                float p[24];
-                const uint32_t rowa = taddr + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * Cfg::NP + grp * 8);
-                tmem_ld8x3(rowa, rowa + (uint32_t)N, rowa + (uint32_t)(2 * N), p);
-                fence_before_sync();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&tempty_b[acc]));
-                // lanes m - 1 and m + 1 are the x-neighbours (same block row for
-                // the interior cells that produce output)
-#pragma unroll
-                for (int o = 0; o < 8; ++o) {
-                    const float left = __shfl_up_sync(0xffffffffu, p[o], 1);
-                    const float right = __shfl_down_sync(0xffffffffu, p[16 + o], 1);
-                    v[o] = left + p[8 + o] + right;
-                }
-            }
-            __nv_bfloat16 *out = a.y ? a.y + obase : nullptr;
-            float *outf = a.y_f32 ? a.y_f32 + obase : nullptr;
-            if (valid) {
-                float r8[8];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    float s = v[j] + bias8[j];
-                    if (a.relu) s = fmaxf(s, 0.0f);
-                    if (a.scale_out) {
-                        const uint32_t f = (keep16[j >> 1] >> (16 * (j & 1))) & 0xFFFFu;
-                        s = f >= a.drop_thr ? s * scale : 0.0f;
+                    for (int j = 0; j < EPC; j += 2) {
+                        const float2 s2 = unpack2(v2[j / 2]);
+                        v[j] = s2.x;
+                        v[j + 1] = s2.y;
                     }
-                    r8[j] = s;
-                }
-                if (outf && a.accum) {
                     // partial sums of one input-channel chunk: add the raw accumulator
-                    float4 *o4 = reinterpret_cast<float4 *>(outf);
-                    const float4 p0 = o4[0], p1 = o4[1];
-                    o4[0] = make_float4(p0.x + v[0], p0.y + v[1], p0.z + v[2], p0.w + v[3]);
-                    o4[1] = make_float4(p1.x + v[4], p1.y + v[5], p1.z + v[6], p1.w + v[7]);
-                } else if (outf) {
-                    reinterpret_cast<float4 *>(outf)[0] = make_float4(r8[0], r8[1], r8[2], r8[3]);
-                    reinterpret_cast<float4 *>(outf)[1] = make_float4(r8[4], r8[5], r8[6], r8[7]);
-                } else {
-                    __align__(16) __nv_bfloat16 o[8];
+                    float4 *o4 = reinterpret_cast<float4 *>(a.y_f32 + obase);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) o[j] = __float2bfloat16_rn(r8[j]);
-                    *reinterpret_cast<uint4 *>(out) = *reinterpret_cast<const uint4 *>(o);
+                    for (int j = 0; j < EPC / 4; ++j) {
+                        const float4 p0 = o4[j];
+                        o4[j] = make_float4(p0.x + v[4 * j], p0.y + v[4 * j + 1], p0.z + v[4 * j + 2], p0.w + v[4 * j + 3]);
+                    }
+                    continue;
+                }
+#pragma unroll
+                for (int j = 0; j < EPC; j += 2) {
+                    float2 s2 = unpack2(add2(v2[j / 2], bias[j / 2]));
+                    if (a.relu) s2 = make_float2(fmaxf(s2.x, 0.0f), fmaxf(s2.y, 0.0f));
+                    s2 = unpack2(mul2(f32x2(s2.x, s2.y), scale2));
+                    v[j] = s2.x;
+                    v[j + 1] = s2.y;
+                }
+                if (a.y_f32) {
+                    float4 *o4 = reinterpret_cast<float4 *>(a.y_f32 + obase);
+#pragma unroll
+                    for (int j = 0; j < EPC; ++j)
+                        if (!((keep[j >> 1] >> (16 * (j & 1))) & 1u)) v[j] = 0.0f;
+#pragma unroll
+                    for (int j = 0; j < EPC / 4; ++j)
+                        o4[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                } else {
+                    uint32_t o[EPC / 2];
+#pragma unroll
+                    for (int j = 0; j < EPC / 2; ++j) {
+                        const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+                        o[j] = *reinterpret_cast<const uint32_t *>(&h) & keep[j];
+                    }
+                    uint4 *o4 = reinterpret_cast<uint4 *>(a.y + obase);
+                    o4[0] = make_uint4(o[0], o[1], o[2], o[3]);
+                    o4[1] = make_uint4(o[4], o[5], o[6], o[7]);
                 }
             }
         }
@@ -373,7 +473,7 @@ __global__ void __launch_bounds__(ConvCfg<KC, N>::NTHREADS, 1)
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
-    if (warp == 1) tmem_dealloc(taddr, Cfg::TCOLS);
+    if (warp == 1) tmem_dealloc(taddr, 512);
 }
 
 // ---------------------------------------------------------------- host side
@@ -397,7 +497,7 @@ static EncodeTiledFn encode_fn() {
 }
 
 // tensor map of a channels-last BF16 activation [B][D][H][W][C]: dims
-// (C, W, H, D, B), box (8 channels, halo x, halo y, halo z, 1)
+// (C, W, H, D, B), box (16 or 32 channels, halo x, halo y, 1 plane, 1)
 static hyb_status make_tmap(CUtensorMap *tm, const ConvArgs &a) {
     EncodeTiledFn enc = encode_fn();
     if (!enc) return set_error(HYB_ECUDA, "cuTensorMapEncodeTiled is not available");
@@ -405,10 +505,10 @@ static hyb_status make_tmap(CUtensorMap *tm, const ConvArgs &a) {
     const cuuint64_t dims[5] = {C, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)a.D, (cuuint64_t)a.B};
     const cuuint64_t es = 2;
     const cuuint64_t strides[4] = {es * C, es * C * a.W, es * C * a.W * a.H, es * C * a.W * a.H * a.D};
-    const cuuint32_t box[5] = {16, (cuuint32_t)TX, (cuuint32_t)HY, (cuuint32_t)HZ, 1};
+    const cuuint32_t box[5] = {(cuuint32_t)a.cin, (cuuint32_t)TX, (cuuint32_t)HY, 1, 1};
     const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
     CUresult r = enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, (void *)a.x, dims, strides, box, estr,
-                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE, a.cin == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return set_error(HYB_ECUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")");
     return HYB_OK;
@@ -422,11 +522,11 @@ static hyb_status launch_cfg(const ConvArgs &a, cudaStream_t st) {
     if (s != HYB_OK) return s;
     // per-device launch set-up, done once (its host cost shows on small grids)
     static std::mutex mu;
-    static int ready_dev[64] = {0}, nsm_dev[64] = {0}, per_sm_dev[64] = {0};
+    static int ready_dev[64] = {0}, nsm_dev[64] = {0};
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) return set_error(HYB_EINVAL, "device index out of range");
-    int nsm, per_sm;
+    int nsm;
     {
         std::lock_guard<std::mutex> lock(mu);
         if (!ready_dev[dev]) {
@@ -435,20 +535,31 @@ static hyb_status launch_cfg(const ConvArgs &a, cudaStream_t st) {
             if (e != cudaSuccess)
                 return set_error(HYB_ECUDA, std::string("conv smem attribute: ") + cudaGetErrorString(e));
             cudaDeviceGetAttribute(&nsm_dev[dev], cudaDevAttrMultiProcessorCount, dev);
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_dev[dev], k_conv3_tc<KC, N>, Cfg::NTHREADS,
-                                                          Cfg::SMEM);
             ready_dev[dev] = 1;
         }
         nsm = nsm_dev[dev];
-        per_sm = per_sm_dev[dev];
     }
     cudaError_t e;
     int tx0, ntx;
     conv_tiles_x(a.W, a.x_lo, a.x_hi, tx0, ntx);
-    const long long ntiles = (long long)a.B * a.D * (a.H / TY) * ntx;
-    if (ntiles == 0) return HYB_OK;
-    const long long grid = std::min<long long>(ntiles, (long long)nsm * std::max(per_sm, 1));
-    k_conv3_tc<KC, N><<<(unsigned)grid, Cfg::NTHREADS, Cfg::SMEM, st>>>(tm, a);
+    // output planes per column: the length that leaves the busiest SM the fewest
+    // planes to compute, a fetched halo plane counted as a fifth of one (its
+    // shared-memory writes against an output plane's MMAs)
+    const long long cols = (long long)a.B * (a.H / TY) * ntx;
+    if (cols == 0) return HYB_OK;
+    ConvArgs b = a;
+    double best = 0.0;
+    for (int lz = 2; lz <= 32; ++lz) {
+        const long long u = cols * ((a.D + lz - 1) / lz);
+        const double t = (double)((u + nsm - 1) / nsm) * (std::min(lz, a.D) + 0.4);
+        if (lz == 2 || t < best) {
+            best = t;
+            b.lz = lz;
+        }
+    }
+    const long long units = cols * ((a.D + b.lz - 1) / b.lz);
+    const long long grid = std::min<long long>(units, (long long)nsm);  // one CTA per SM (all of its TMEM)
+    k_conv3_tc<KC, N><<<(unsigned)grid, Cfg::NTHREADS, Cfg::SMEM, st>>>(tm, b);
     e = cudaGetLastError();
     if (e != cudaSuccess) return set_error(HYB_ECUDA, std::string("conv launch: ") + cudaGetErrorString(e));
     return HYB_OK;

@@ -42,6 +42,18 @@ __device__ __forceinline__ uint64_t smem_desc_sw32(uint32_t addr, uint32_t sbo) 
     return d;
 }
 
+// the same with rows of 64 bytes (32 BF16 along K) and the 64-byte swizzle
+// (layout type 4); a 16-channel block starts 32 bytes into the row
+__device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t addr, uint32_t sbo) {
+    uint64_t d = 0;
+    d |= (uint64_t)((addr >> 4) & 0x3FFFu);
+    d |= (uint64_t)1 << 16;
+    d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)4 << 61;
+    return d;
+}
+
 // instruction descriptor for kind::f16: FP32 accumulator (bits [4,6) = 1),
 // BF16 A and B (bits [7,10) = 1, [10,13) = 1), both K-major, N>>3 in
 // [17,23), M>>4 in [24,29)
@@ -66,6 +78,28 @@ __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint6
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
+}
+
+// The same issued by one elected lane of a warp whose lanes all run the issue
+// loop on equal values: descriptors and addresses then stay in uniform
+// registers.  Issued by a lone lane (a divergent branch) every operand is moved
+// there first, about 80 cycles an instruction -- more than the MMA takes.
+// The descriptors' upper words (strides, layout) are constant.
+__device__ __forceinline__ void umma_bf16_warp(uint32_t tmem_d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
+                                               uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\t"
+        "mov.b64 da, {%1, %2};\n\tmov.b64 db, {%3, %4};\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}\n" ::"r"(tmem_d),
+        "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate));
+}
+__device__ __forceinline__ void umma_commit_warp(uint32_t mbar_smem) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n" ::"r"(mbar_smem)
+        : "memory");
 }
 
 __device__ __forceinline__ void umma_commit(uint32_t mbar_smem) {
@@ -98,6 +132,100 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, long l
     return false;
 }
 
+// the same, giving up at once when another role has (the flag is only read
+// while waiting)
+__device__ __forceinline__ bool mbar_wait_abort(uint32_t mbar, uint32_t parity, long long limit, const int *abort_flag) {
+    for (long long it = 0; it < limit; ++it) {
+        uint32_t done;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.b32 %0, 1, 0, p;\n\t}\n"
+            : "=r"(done)
+            : "r"(mbar), "r"(parity)
+            : "memory");
+        if (done) return true;
+        if (*(const volatile int *)abort_flag) return false;
+    }
+    return false;
+}
+
+// whether the phase `parity` of an mbarrier has completed (one poll)
+__device__ __forceinline__ bool mbar_test(uint32_t mbar, uint32_t parity) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.b32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(done)
+        : "r"(mbar), "r"(parity)
+        : "memory");
+    return done != 0;
+}
+
+// The waits of an MMA-issuing warp.  A wait on a barrier that has completed
+// still costs some 200 cycles before the next instruction, more than the queue
+// of issued MMAs covers, so the warp looks ahead: lanes 0-7 poll the next eight
+// entries of one ring (S entries: operands that arrived), lanes 8-15 the next
+// entries of another (R entries: accumulators that were drained), all in one
+// instruction, and the entries found ready are used without another wait.
+// `limit` polls bound the wait; it ends early when another role gave up.
+template <int S, int R>
+struct LookAhead {
+    int nf = 0, ne = 0;  // entries known to be ready
+    // entry f (phase parity fp) of the first ring, and entry e (parity ep) of the second unless !need_e
+    __device__ __forceinline__ bool wait(const uint64_t *full, int f, uint32_t fp, const uint64_t *empty, int e,
+                                         uint32_t ep, bool need_e, int lane, long long limit, const int *abort_flag) {
+        constexpr int LS = S < 8 ? S : 8, LR = R < 8 ? R : 8;
+        for (long long it = 0; nf == 0 || (need_e && ne == 0); ++it) {
+            if (it >= limit || (it > 0 && *(const volatile int *)abort_flag)) return false;
+            int i = f + (lane & 7);
+            uint32_t par = fp;
+            const uint64_t *bar = full;
+            if (lane & 8) {
+                i = e + (lane & 7);
+                par = ep;
+                bar = empty;
+            }
+            const int n = lane & 8 ? R : S;
+            if (i >= n) {
+                i -= n;
+                par ^= 1;
+            }
+            const bool in = (lane & 7) < (lane & 8 ? LR : LS);
+            const unsigned m = __ballot_sync(0xffffffffu, in && mbar_test(smem_u32(bar + (in ? i : 0)), par));
+            nf = __ffs((int)~(m & 0xFFu)) - 1;
+            ne = __ffs((int)~((m >> 8) & 0xFFu)) - 1;
+            __syncwarp();
+        }
+        --nf;
+        if (need_e) --ne;
+        return true;
+    }
+};
+
+// two FP32 additions or products in one instruction, each rounded as alone
+__device__ __forceinline__ uint64_t f32x2(float lo, float hi) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t a) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+    return r;
+}
+
 // plain arrival (count 1) on an mbarrier
 __device__ __forceinline__ void mbar_arrive(uint32_t mbar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mbar) : "memory");
@@ -122,37 +250,37 @@ __device__ __forceinline__ void tma_load_5d(uint32_t dst, const void *tmap, int 
         : "memory");
 }
 
+// untiled bulk copy global -> shared (both 16-byte aligned, bytes a multiple of
+// 16), completion counted on mbar
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t mbar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "l"(src), "r"(bytes), "r"(mbar)
+                 : "memory");
+}
+
 __device__ __forceinline__ void prefetch_tmap(const void *tmap) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(tmap) : "memory");
 }
 
-// 32 lanes x 32 bits, 8 consecutive columns
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float v[8]) {
-    uint32_t r[8];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// three loads of 32 lanes x 32 bits x 8 consecutive columns (at t0, t1, t2)
-// under one wait: v[8 k + i] = column i of load k
-__device__ __forceinline__ void tmem_ld8x3(uint32_t t0, uint32_t t1, uint32_t t2, float v[24]) {
-    uint32_t r[24];
+// three loads of 32 lanes x 32 bits x 16 consecutive columns (at t0, t1, t2)
+// under one wait: v[16 k + i] = column i of load k
+__device__ __forceinline__ void tmem_ld16x3(uint32_t t0, uint32_t t1, uint32_t t2, float v[48]) {
+    uint32_t r[48];
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%24];\n\t"
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%25];\n\t"
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%16,%17,%18,%19,%20,%21,%22,%23}, [%26];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%48];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%49];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%32,%33,%34,%35,%36,%37,%38,%39,%40,%41,%42,%43,%44,%45,%46,%47}, [%50];\n\t"
         "tcgen05.wait::ld.sync.aligned;"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23])
+          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]),
+          "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]),
+          "=r"(r[40]), "=r"(r[41]), "=r"(r[42]), "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47])
         : "r"(t0), "r"(t1), "r"(t2)
         : "memory");
 #pragma unroll
-    for (int i = 0; i < 24; ++i) v[i] = __uint_as_float(r[i]);
+    for (int i = 0; i < 48; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 // 32 lanes x 32 bits, 32 consecutive columns under one wait
@@ -211,6 +339,7 @@ struct ConvArgs {
     uint32_t seed, pass, layer;
     int *status;
     int x_lo, x_hi;           // when x_hi > x_lo: only the tiles whose outputs meet x_lo <= x < x_hi
+    int lz;                   // output planes per column of blocks (set by the launch)
 };
 hyb_status launch_conv3_tc(const ConvArgs &a, cudaStream_t st);
 
