@@ -775,7 +775,6 @@ static hyb_status layer_wgrad(hyb_model *m, TrainBufs &t, int l, const __nv_bflo
     j.x = A;
     j.x_pitch = ca;
     j.ci_n = CIN[l];
-    j.ci_tot = CIN[l];
     j.dz = dZ;
     j.dz_f32 = dZf;
     j.dz_pitch = COUT[l];

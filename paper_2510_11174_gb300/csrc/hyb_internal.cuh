@@ -434,18 +434,19 @@ __global__ void k_loss(const float *__restrict__ logit, const float *__restrict_
                        float inv_emean, float lam, long long n, float *__restrict__ dlogit, double *__restrict__ part);
 
 // ---------------------------------------------------------------- weight gradients on the tensor cores (wgrad_tc.cu)
-// dW[co0 + co][ci0 + ci][t] = sum over cells of dZ[cell][co0 + co] X[cell + s(t)][ci0 + ci]
-// for a 3x3x3 convolution (taps = 27, zero outside the volume) or a dense
-// layer (taps = 1); co_n <= 32 (conv) or <= 128 (dense), ci_n <= 32 (conv) or
-// <= 256 (dense).  gw has the layout [co][ci_tot][taps]; gb (optional) gets
-// sum over cells of dZ.  dZ is BF16 channels-last [cells][dz_pitch], or FP32
-// [cells] with one channel (dz_f32, conv only).  Deterministic.
+// dW[co][ci][t] = sum over cells of dZ[cell][co] X[cell + s(t)][ci] for a whole
+// 3x3x3 convolution (taps = 27, zero outside the volume) or dense layer (taps =
+// 1).  X and dZ are BF16 channels-last with pitches padded to 16 (convolution),
+// or 128 outputs and 16, 128 or 256 inputs (dense); the padding channels are
+// not written.  gw has the layout [co][ci][taps]; gb (optional) gets the sum
+// over cells of dZ.  dz_f32: FP32 [cells] with one channel instead of dZ
+// (convolution only; its weight gradient takes the BF16 values).  Deterministic.
 struct WgradJob {
     const __nv_bfloat16 *x;  // [cells][x_pitch]
-    int x_pitch, ci0, ci_n, ci_tot;
+    int x_pitch, ci_n;
     const __nv_bfloat16 *dz;  // [cells][dz_pitch]
     const float *dz_f32;
-    int dz_pitch, co0, co_n;
+    int dz_pitch, co_n;
     int B, D, H, W;           // dense: B = D = H = 1, W = rows
     int taps;
     float *gw, *gb;

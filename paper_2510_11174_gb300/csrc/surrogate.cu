@@ -10,7 +10,7 @@
 // finishing kernel adds the bias, applies ReLU, dropout and the identity
 // shortcut, and stores the BF16 activation.  The data gradient is the same
 // convolution with the transposed, flipped kernel; the weight gradient is the
-// tensor-core contraction over the cells (wgrad_tc) in blocks of 32 x 32 channels;
+// tensor-core contraction over the cells (wgrad_tc);
 // Adam updates FP32 masters.  See hyb_surrogate_* in include/hyb.h.
 #include <cuda_bf16.h>
 
@@ -295,15 +295,6 @@ __global__ void k_sur_pack(const float *__restrict__ W, int ci_n, int co_n, int 
     out[t] = __float2bfloat16_rn(v);
 }
 
-// summed weight-gradient block [tap][ci][co] (ci_n x co_n) -> gw[co0 + co][ci0 + ci][tap]
-__global__ void k_sur_scatter_wg(const float *__restrict__ in, int ci_n, int co_n, int ci0, int co0, int CItot,
-                                 float *__restrict__ gw) {
-    const int o = blockIdx.x * blockDim.x + threadIdx.x;
-    if (o >= 27 * ci_n * co_n) return;
-    const int co = o % co_n, ci = (o / co_n) % ci_n, tap = o / (co_n * ci_n);
-    gw[((long long)(co0 + co) * CItot + ci0 + ci) * 27 + tap] = in[o];
-}
-
 }  // namespace
 }  // namespace hyb
 
@@ -466,33 +457,25 @@ hyb_status read_status(hyb_surrogate *m) {
 }
 
 // weight and bias gradient of layer l on the tensor cores, from its input
-// a[l] and the BF16 data gradient dz, in blocks of 32 x 32 channels
+// a[l] and the BF16 data gradient dz
 hyb_status layer_wgrad(hyb_surrogate *m, int l, int B, int D, int H, int W) {
-    for (int ci0 = 0; ci0 < CI[l]; ci0 += 32)
-        for (int co0 = 0; co0 < CO[l]; co0 += 32) {
-            WgradJob j;
-            memset(&j, 0, sizeof(j));
-            j.x = m->a[l];
-            j.x_pitch = CIP[l];
-            j.ci0 = ci0;
-            j.ci_n = CI[l] - ci0 < 32 ? CI[l] - ci0 : 32;
-            j.ci_tot = CI[l];
-            j.dz = m->dz;
-            j.dz_pitch = COP[l];
-            j.co0 = co0;
-            j.co_n = CO[l] - co0 < 32 ? CO[l] - co0 : 32;
-            j.B = B;
-            j.D = D;
-            j.H = H;
-            j.W = W;
-            j.taps = 27;
-            j.gw = m->gw[l];
-            j.gb = ci0 == 0 ? m->gb[l] : nullptr;
-            j.status = m->status;
-            hyb_status s = wgrad_tc(j, *m->wg, m->stream);
-            if (s != HYB_OK) return s;
-        }
-    return HYB_OK;
+    WgradJob j;
+    memset(&j, 0, sizeof(j));
+    j.x = m->a[l];
+    j.x_pitch = CIP[l];
+    j.ci_n = CI[l];
+    j.dz = m->dz;
+    j.dz_pitch = COP[l];
+    j.co_n = CO[l];
+    j.B = B;
+    j.D = D;
+    j.H = H;
+    j.W = W;
+    j.taps = 27;
+    j.gw = m->gw[l];
+    j.gb = m->gb[l];
+    j.status = m->status;
+    return wgrad_tc(j, *m->wg, m->stream);
 }
 
 }  // namespace

@@ -517,17 +517,15 @@ hyb_status hyb_switchnet_train_step(hyb_switchnet *m, const float *x, const floa
         if (l < SN_L - 1)
             k_act_dz<<<nbs(n * (SN_CO[l] / 8)), RBS, 0, st>>>(G, m->z[l], m->b[l], SN_CO[l], SN_RELU[l],
                                                               sn_drop(m, l, pass), 1, n, m->dz);
-        for (int co0 = 0; co0 < SN_CO[l]; co0 += 128) {
+        {
             WgradJob j;
             memset(&j, 0, sizeof(j));
             j.x = m->a[l];
             j.x_pitch = SN_KP[l];
             j.ci_n = SN_CI[l];
-            j.ci_tot = SN_CI[l];
             j.dz = m->dz;
             j.dz_pitch = SN_CO[l];
-            j.co0 = co0;
-            j.co_n = 128;
+            j.co_n = SN_CO[l];
             j.B = j.D = j.H = 1;
             j.W = (int)n;
             j.taps = 1;
