@@ -22,15 +22,15 @@
 // where out-of-volume cells are 0 (TMA fill).  A is dZ (taps (sz, 2 - sy, dx)) or
 // X (taps (2 - sz, sy, 2 - dx)), whichever has 32 channels.
 // A CTA walks columns of 16 (x) x 8 (y) cells along z with rings of planes of
-// both operands, keeps its 3 x 3 CB accumulator columns in TMEM throughout and
-// writes them once at the end; the partial sums of a channel block's CTAs are
+// both operands and 3 x 3 CB accumulator columns in TMEM; the partial sums of a channel block's CTAs are
 // added in a fixed order (deterministic).
 // Dense layer (k_wgrad_dense): the same with plain 64-cell tiles, M = 128 output
 // columns, N = 16, 128 or 256 input columns.
 //   warp 0      TMA producer;
 //   warp 1      MMA issuer;
-//   warps 2..5  epilogue at the end of the CTA's range: tcgen05.ld of every
-//               accumulator, FP32 partials to global memory.
+//   warps 2..17 epilogue: tcgen05.ld of the accumulators into FP32 register sums
+//               (see wg_epilogue), FP32 partials to global memory at the end of
+//               the CTA's range.
 // What bounds the convolution: fetching the operands from shared memory, 56
 // cycles per 128 x 96 x 16 MMA (48 of math), 10.5 cycles a cell.  The former
 // kernel wanted [16 positions][channel] transposes of both operands over the
@@ -71,6 +71,7 @@ struct WgConvArgs {
     int B, D, H, W;
     int nab;                   // channel blocks of A (block = ab + nab * bb)
     int lz;                    // planes per column
+    int flush;                 // planes (8 K-steps each) the accumulators hold before they are taken over
     int *status;
 };
 
@@ -101,34 +102,76 @@ __device__ __forceinline__ void wg_unit(long long u, const WgConvArgs &a, int nx
     z1 = min(z0 + a.lz, a.D);
 }
 
-// the accumulators of a CTA's range as FP32 partials, [column][128 rows]
-// (zeros where the range was empty)
-template <int COLS>
-__device__ __forceinline__ void wg_store(uint32_t taddr, int warp, int lane, bool any, float *__restrict__ dst) {
-    const int q = warp & 3, row = q * 32 + lane;
-#pragma unroll 1
-    for (int c0 = 0; c0 < COLS; c0 += 16) {
-        float v[16];
-        if (any) {
-            tmem_ld16(taddr + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, v);
-        } else {
+// The tensor core's FP32 accumulation truncates, so a sum's error grows with the
+// number of products added in place (a 64 -> 128 layer over 131,072 cells: 9e-6
+// off after 431, 3e-7 after 64).  Where channel blocks share the SMs a CTA has
+// more than the 1 / (number of SMs) of the cells it would have alone: the 16
+// epilogue warps take the accumulators over after every such share and add
+// them, rounded to nearest, to registers; warp w of a lane quarter keeps COLS / 4
+// columns.
+static constexpr int WG_EPI = 16;
+static constexpr int WG_THREADS = 64 + 32 * WG_EPI;
+
+// 32 lanes x 32 bits x G consecutive columns, without a wait
+template <int G>
+__device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, float (&v)[G]) {
+    uint32_t r[G];
+    if constexpr (G == 8)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                     : "r"(taddr));
+    else
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                     : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-            for (int k = 0; k < 16; ++k) v[k] = 0.0f;
+    for (int i = 0; i < G; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// `flushes` rounds: wait for the accumulators (columns from taddr; BUF buffers
+// of `pitch` columns in turn), add them, hand them back; then the sums as
+// partials [column][128 rows].  false: a wait gave up.
+template <int COLS, int BUF>
+__device__ __forceinline__ bool wg_epilogue(uint32_t taddr, int pitch, uint64_t *full, uint64_t *empty, long long flushes,
+                                            int warp, int lane, const int *abort_flag, float *__restrict__ dst) {
+    constexpr int CPW = COLS / 4, G = CPW % 8 == 0 ? 8 : 4;
+    const int q = warp & 3, w = (warp - 2) >> 2;
+    float acc[CPW];
+#pragma unroll
+    for (int k = 0; k < CPW; ++k) acc[k] = 0.0f;
+    for (long long i = 0; i < flushes; ++i) {
+        const int b = (int)(i % BUF);
+        const bool ok = mbar_wait_abort(smem_u32(&full[b]), (uint32_t)(i / BUF) & 1u, WG_MBAR_LIMIT, abort_flag);
+        if (!__all_sync(0xffffffffu, ok)) return false;
+        fence_after_sync();
+        const uint32_t t = taddr + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * pitch + w * CPW);
+#pragma unroll
+        for (int c = 0; c < CPW; c += G) {
+            float v[G];
+            tmem_ld_cols<G>(t + (uint32_t)c, v);
+#pragma unroll
+            for (int k = 0; k < G; ++k) acc[c + k] += v[k];
         }
-#pragma unroll
-        for (int k = 0; k < 16; ++k) dst[(c0 + k) * WROWS + row] = v[k];
+        fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&empty[b]));
     }
+    const int row = q * 32 + lane;
+#pragma unroll
+    for (int k = 0; k < CPW; ++k) dst[(w * CPW + k) * WROWS + row] = acc[k];
+    return true;
 }
 
 template <int CA, int CB>
-__global__ void __launch_bounds__(192, 1) k_wgrad_conv(const __grid_constant__ CUtensorMap ta,
+__global__ void __launch_bounds__(WG_THREADS, 1) k_wgrad_conv(const __grid_constant__ CUtensorMap ta,
                                                        const __grid_constant__ CUtensorMap tb,
                                                        const __grid_constant__ WgConvArgs a) {
     using Cfg = WgConv<CA, CB>;
     constexpr int NA = Cfg::NA, NB = Cfg::NB;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    __shared__ __align__(8) uint64_t fa_b[NA], ea_b[NA], fb_b[NB], eb_b[NB], done_b;
+    __shared__ __align__(8) uint64_t fa_b[NA], ea_b[NA], fb_b[NB], eb_b[NB], tfull_b, tempty_b, done_b;
     __shared__ uint32_t taddr_s;
     __shared__ int abort_s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -145,6 +188,8 @@ __global__ void __launch_bounds__(192, 1) k_wgrad_conv(const __grid_constant__ C
             mbar_init(smem_u32(&fb_b[s]), 1);
             mbar_init(smem_u32(&eb_b[s]), 1);
         }
+        mbar_init(smem_u32(&tfull_b), 1);
+        mbar_init(smem_u32(&tempty_b), WG_EPI);
         mbar_init(smem_u32(&done_b), 1);
         abort_s = 0;
         fence_mbar_init();
@@ -228,6 +273,8 @@ __global__ void __launch_bounds__(192, 1) k_wgrad_conv(const __grid_constant__ C
         int s = 0, t = 0;        // A plane, next B plane to wait for
         uint32_t ps = 0, pt = 0;
         uint32_t acc = 0;        // 0: the first products overwrite the accumulators
+        int planes = 0;          // planes in the accumulators
+        uint32_t pf = 0;         // parity of the last hand-over
         LookAhead<NB, NA> look;
         bool stop = false;
         for (long long u = blockIdx.x; u < nunits && !stop; u += gridDim.x) {
@@ -246,6 +293,19 @@ __global__ void __launch_bounds__(192, 1) k_wgrad_conv(const __grid_constant__ C
                     pt ^= 1;
                 }
                 if (z <= z0) continue;
+                if (planes == a.flush) {
+                    // hand the accumulators over and begin again
+                    umma_commit_warp(smem_u32(&tfull_b));
+                    if (!__all_sync(0xffffffffu, mbar_wait_abort(smem_u32(&tempty_b), pf, WG_MBAR_LIMIT, &abort_s))) {
+                        if (lane == 0) fail();
+                        stop = true;
+                        break;
+                    }
+                    pf ^= 1;
+                    planes = 0;
+                    acc = 0;
+                }
+                ++planes;
                 fence_after_sync();
                 const int n1 = min(3, NB - first);   // planes before the ring wraps
                 const uint32_t ap = alo + (uint32_t)(s * (Cfg::ABOX >> 4));
@@ -266,9 +326,10 @@ __global__ void __launch_bounds__(192, 1) k_wgrad_conv(const __grid_constant__ C
                             const uint32_t ad = ap + (uint32_t)((j * Cfg::AROW) >> 4);
                             const uint32_t off = (uint32_t)((j * Cfg::BROW + dx * CB * 2) >> 4);
                             const uint32_t d = taddr + (uint32_t)(dx * 3 * CB);
-                            umma_bf16_warp(d, ad, ahi, bp + off, bhi, idesc_mn(8) - (1u << 17) + ((uint32_t)(n1 * CB) << 14), 1);
+                            umma_bf16_warp(d, ad, ahi, bp + off, bhi, idesc_mn(8) - (1u << 17) + ((uint32_t)(n1 * CB) << 14),
+                                           acc | (uint32_t)j);
                             umma_bf16_warp(d + (uint32_t)(n1 * CB), ad, ahi, blo + off, bhi,
-                                           idesc_mn(8) - (1u << 17) + ((uint32_t)((3 - n1) * CB) << 14), 1);
+                                           idesc_mn(8) - (1u << 17) + ((uint32_t)((3 - n1) * CB) << 14), acc | (uint32_t)j);
                         }
                 }
                 acc = 1;
@@ -286,18 +347,20 @@ __global__ void __launch_bounds__(192, 1) k_wgrad_conv(const __grid_constant__ C
                 }
             }
         }
+        if (planes) umma_commit_warp(smem_u32(&tfull_b));
         umma_commit_warp(smem_u32(&done_b));
         mbar_wait(smem_u32(&done_b), 0, WG_MBAR_LIMIT);
     } else {
-        // epilogue: the accumulators once every MMA of the range has completed
-        const bool ok = mbar_wait(smem_u32(&done_b), 0, WG_MBAR_LIMIT);
-        if (!__all_sync(0xffffffffu, ok) || *(volatile int *)&abort_s) {
-            if (lane == 0) atomicOr(a.status, ST_TIMEOUT);
-        } else {
-            fence_after_sync();
-            wg_store<Cfg::COLS>(taddr, warp, lane, (long long)blockIdx.x < nunits,
-                                a.part + ((long long)blockIdx.y * gridDim.x + blockIdx.x) * Cfg::COLS * WROWS);
+        long long total = 0;     // planes of this CTA's columns
+        for (long long u = blockIdx.x; u < nunits; u += gridDim.x) {
+            int x, y, z0, z1, b;
+            wg_unit(u, a, nx, ny, nzc, x, y, z0, z1, b);
+            total += z1 - z0;
         }
+        if (!wg_epilogue<Cfg::COLS, 1>(taddr, 0, &tfull_b, &tempty_b, (total + a.flush - 1) / a.flush, warp, lane, &abort_s,
+                                       a.part + ((long long)blockIdx.y * gridDim.x + blockIdx.x) * Cfg::COLS * WROWS) &&
+            lane == 0)
+            fail();
     }
     fence_before_sync();
     __syncthreads();
@@ -310,6 +373,7 @@ __global__ void __launch_bounds__(192, 1) k_wgrad_conv(const __grid_constant__ C
 struct WgDenseArgs {
     float *part;      // [co slice][cta][N columns][128 rows]
     long long tiles;  // of 64 cells
+    int flush;        // tiles the accumulators hold before they are taken over
     int *status;
 };
 
@@ -331,25 +395,29 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const void *tmap, int 
 }
 
 template <int N>
-__global__ void __launch_bounds__(192, 1) k_wgrad_dense(const __grid_constant__ CUtensorMap tz,
+__global__ void __launch_bounds__(WG_THREADS, 1) k_wgrad_dense(const __grid_constant__ CUtensorMap tz,
                                                         const __grid_constant__ CUtensorMap tx,
                                                         const __grid_constant__ WgDenseArgs a) {
     using Cfg = WgDense<N>;
     constexpr int STAGES = Cfg::STAGES;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *ring = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    __shared__ __align__(8) uint64_t full_b[STAGES], empty_b[STAGES], done_b;
+    __shared__ __align__(8) uint64_t full_b[STAGES], empty_b[STAGES], tfull_b[2], tempty_b[2], done_b;
     __shared__ uint32_t taddr_s;
     __shared__ int abort_s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (warp == 1) {
-        tmem_alloc(smem_u32(&taddr_s), 256);
+        tmem_alloc(smem_u32(&taddr_s), 512);
         tmem_relinquish();
     }
     if (tid == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(smem_u32(&full_b[s]), 1);
             mbar_init(smem_u32(&empty_b[s]), 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(smem_u32(&tfull_b[b]), 1);
+            mbar_init(smem_u32(&tempty_b[b]), WG_EPI);
         }
         mbar_init(smem_u32(&done_b), 1);
         abort_s = 0;
@@ -399,13 +467,24 @@ __global__ void __launch_bounds__(192, 1) k_wgrad_dense(const __grid_constant__ 
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            int s = 0;
-            uint32_t ph = 0, acc = 0;
+            // two accumulator buffers in turn, a.flush tiles each
+            int s = 0, tiles = 0, buf = 0;
+            uint32_t ph = 0, acc = 0, pb = 1;
             for (long long k = blockIdx.x; k < a.tiles; k += gridDim.x) {
-                if (!mbar_wait(smem_u32(&full_b[s]), ph, WG_MBAR_LIMIT) || *(volatile int *)&abort_s) {
+                if (tiles == a.flush) {
+                    umma_commit(smem_u32(&tfull_b[buf]));
+                    buf ^= 1;
+                    if (buf == 0) pb ^= 1;
+                    tiles = 0;
+                    acc = 0;
+                }
+                if ((tiles == 0 && !mbar_wait_abort(smem_u32(&tempty_b[buf]), pb, WG_MBAR_LIMIT, &abort_s)) ||
+                    !mbar_wait_abort(smem_u32(&full_b[s]), ph, WG_MBAR_LIMIT, &abort_s)) {
                     fail();
+                    tiles = 0;
                     break;
                 }
+                ++tiles;
                 fence_after_sync();
                 const uint32_t st = ring_s + (uint32_t)(s * Cfg::STAGE);
                 const uint64_t ad = smem_desc_mn(st, 8192, 1024, SW128);
@@ -413,7 +492,7 @@ __global__ void __launch_bounds__(192, 1) k_wgrad_dense(const __grid_constant__ 
                                            : smem_desc_mn(st + Cfg::ABYTES, 8192, 1024, SW128);
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) {
-                    umma_bf16(taddr, ad + (uint64_t)((kk * 16 * 128) >> 4),
+                    umma_bf16(taddr + (uint32_t)(buf * 256), ad + (uint64_t)((kk * 16 * 128) >> 4),
                               bd + (uint64_t)((kk * 16 * Cfg::BW * 2) >> 4), idesc_mn(N), acc);
                     acc = 1;
                 }
@@ -423,23 +502,21 @@ __global__ void __launch_bounds__(192, 1) k_wgrad_dense(const __grid_constant__ 
                     ph ^= 1;
                 }
             }
+            if (tiles) umma_commit(smem_u32(&tfull_b[buf]));
             umma_commit(smem_u32(&done_b));
             mbar_wait(smem_u32(&done_b), 0, WG_MBAR_LIMIT);
         }
     } else {
-        const bool ok = mbar_wait(smem_u32(&done_b), 0, WG_MBAR_LIMIT);
-        if (!__all_sync(0xffffffffu, ok) || *(volatile int *)&abort_s) {
-            if (lane == 0) atomicOr(a.status, ST_TIMEOUT);
-        } else {
-            fence_after_sync();
-            wg_store<N>(taddr, warp, lane, (long long)blockIdx.x < a.tiles,
-                        a.part + ((long long)blockIdx.y * gridDim.x + blockIdx.x) * N * WROWS);
-        }
+        const long long total = (long long)blockIdx.x < a.tiles ? (a.tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+        if (!wg_epilogue<N, 2>(taddr, 256, tfull_b, tempty_b, (total + a.flush - 1) / a.flush, warp, lane, &abort_s,
+                               a.part + ((long long)blockIdx.y * gridDim.x + blockIdx.x) * N * WROWS) &&
+            lane == 0)
+            fail();
     }
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
-    if (warp == 1) tmem_dealloc(taddr, 256);
+    if (warp == 1) tmem_dealloc(taddr, 512);
 }
 
 // The CTAs' partials of one accumulator column added in a fixed order: 128 rows
@@ -604,7 +681,7 @@ static hyb_status wg_launch(K kern, int smem, const CUtensorMap &m0, const CUten
                             cudaStream_t st) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return set_error(HYB_ECUDA, std::string("wgrad smem attribute: ") + cudaGetErrorString(e));
-    kern<<<grid, 192, smem, st>>>(m0, m1, a);
+    kern<<<grid, WG_THREADS, smem, st>>>(m0, m1, a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return set_error(HYB_ECUDA, std::string("wgrad launch: ") + cudaGetErrorString(e));
     return HYB_OK;
@@ -696,6 +773,7 @@ hyb_status wgrad_tc(const WgradJob &j, WgradScratch &ws, cudaStream_t st) {
         ca.H = j.H;
         ca.W = j.W;
         ca.nab = r.nab;
+        ca.flush = (int)((cells + 128LL * nsm - 1) / (128LL * nsm));
         ca.status = j.status;
         s = vol_map(&ta, r.a_is_dz ? dz : j.x, r.a_is_dz ? zp : xp, j, r.ca, WX, WY + 2);
         if (s == HYB_OK) s = vol_map(&tb, r.a_is_dz ? j.x : dz, r.a_is_dz ? xp : zp, j, r.cb, WX + 2, WY);
@@ -707,6 +785,7 @@ hyb_status wgrad_tc(const WgradJob &j, WgradScratch &ws, cudaStream_t st) {
         WgDenseArgs d;
         d.part = ws.part;
         d.tiles = work;
+        d.flush = (int)((work + nsm - 1) / nsm);
         d.status = j.status;
         s = row_map(&ta, dz, zp, cells, 64);
         if (s == HYB_OK) s = row_map(&tb, j.x, xp, cells, xp < 64 ? 16 : 64);
