@@ -11,7 +11,8 @@
 // tile read from shared memory feeds three times the math.  The epilogue adds
 // the three partial sums of neighbouring x cells (lanes m - 1, m, m + 1, one
 // warp shuffle each way), so a block yields its 14 (x) x 8 (y) interior
-// outputs; blocks step by 14 cells in x.
+// outputs (16 where the volume begins and ends in it); blocks step by 14 cells
+// in x.
 // A CTA walks a column of blocks along z: each plane of the halo (16 x 10
 // cells, all channels) is fetched once by TMA into a ring of planes and used by
 // the three output planes it touches.  With 16 outputs the three z-taps go into
@@ -75,18 +76,21 @@ __host__ __device__ inline bool dropout_keep(uint32_t seed, uint32_t pass, uint3
     return f >= thr;
 }
 
-// the tile columns (x) a launch covers: all, or those whose 14 outputs per
-// row meet the requested x-range
+// Tile t covers the cells 14 t .. 14 t + 15 of a row and yields the outputs that
+// have both x-neighbours in it, plus the volume's first and last cell, whose
+// missing neighbour is 0: ceil((W - 2) / 14) tiles, one for 16 cells (a patch
+// of the surrogate) instead of two.  A launch covers all tile columns, or those
+// whose outputs meet the requested x-range.
 __host__ __device__ inline void conv_tiles_x(int W, int x_lo, int x_hi, int &tx0, int &ntx) {
-    const int all = (W + TXO - 1) / TXO;
+    const int all = W <= TX ? 1 : (W - 2 + TXO - 1) / TXO;
+    tx0 = 0;
+    ntx = all;
     if (x_hi > x_lo) {
-        tx0 = x_lo / TXO;
-        const int tx1 = (x_hi + TXO - 1) / TXO;
-        ntx = (tx1 < all ? tx1 : all) - tx0;
+        const int last = x_hi < 2 ? 0 : (x_hi - 2) / TXO;
+        tx0 = x_lo < 1 ? 0 : (x_lo - 1) / TXO;
+        if (tx0 > all - 1) tx0 = all - 1;
+        ntx = (last < all - 1 ? last : all - 1) - tx0 + 1;
         if (ntx < 0) ntx = 0;
-    } else {
-        tx0 = 0;
-        ntx = all;
     }
 }
 
@@ -138,7 +142,9 @@ struct ConvCfg {
     static constexpr int NTHREADS = 64 + 512;          // producer, MMA issuer, epilogue
 };
 
-template <int KC, int N>
+// EXT: the launch sums over input-channel chunks, adds a shortcut or runs
+// several MC passes side by side (the epilogue without them has no spills)
+template <int KC, int N, bool EXT>
 __global__ void __launch_bounds__(ConvCfg<KC, N>::NTHREADS, 1)
     k_conv3_tc(const __grid_constant__ CUtensorMap tmap, ConvArgs a) {
     using Cfg = ConvCfg<KC, N>;
@@ -150,10 +156,13 @@ __global__ void __launch_bounds__(ConvCfg<KC, N>::NTHREADS, 1)
     uint8_t *wsm = smem;
     uint8_t *ring = smem + Cfg::RING;
     __shared__ __align__(8) uint64_t full_b[PLANES], empty_b[PLANES], tfull_b[NACC], tempty_b[NACC], wfull_b, done_b;
+    __shared__ __align__(16) float bias_s[N];
     __shared__ uint32_t taddr_s;
     __shared__ int abort_s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
+    if (tid >= 64 && tid < 64 + N)
+        bias_s[tid - 64] = a.bias ? __ldg(a.bias + a.out_off + (int)(blockIdx.x % (unsigned)a.nslice) * N + tid - 64) : 0.0f;
     if (warp == 1) {
         tmem_alloc(smem_u32(&taddr_s), 512);
         tmem_relinquish();
@@ -176,14 +185,14 @@ __global__ void __launch_bounds__(ConvCfg<KC, N>::NTHREADS, 1)
         // are in core layout [9 (dz, dy)][KC][NP] already, with ZN = 3 the rows of the
         // three dz of one dy go side by side, dz = 2 (the plane below) first
         const uint32_t wb = smem_u32(&wfull_b), w0 = smem_u32(wsm);
+        const char *wt = reinterpret_cast<const char *>(a.wt) + (blockIdx.x % (unsigned)a.nslice) * Cfg::WBYTES;
         mbar_arrive_expect_tx(wb, Cfg::WBYTES);
         if (ZN == 1) {
-            bulk_load(w0, a.wt, Cfg::WBYTES, wb);
+            bulk_load(w0, wt, Cfg::WBYTES, wb);
         } else {
-            const char *src = reinterpret_cast<const char *>(a.wt);
             for (int i = 0; i < 9 * KC; ++i) {
                 const int z = i % 3, kc = (i / 3) % KC, dy = i / (3 * KC);
-                bulk_load(w0 + (uint32_t)(i * NP * 16), src + (((2 - z) * 3 + dy) * KC + kc) * NP * 16, NP * 16, wb);
+                bulk_load(w0 + (uint32_t)(i * NP * 16), wt + (((2 - z) * 3 + dy) * KC + kc) * NP * 16, NP * 16, wb);
             }
         }
     }
@@ -195,6 +204,9 @@ __global__ void __launch_bounds__(ConvCfg<KC, N>::NTHREADS, 1)
     conv_tiles_x(a.W, a.x_lo, a.x_hi, tx0, tiles_x);
     const int tiles_y = a.H / TY, nzc = (a.D + a.lz - 1) / a.lz;
     const long long nunits = (long long)a.B * nzc * tiles_y * tiles_x;
+    // the CTAs of a launch share its output slices: slice = blockIdx.x % nslice
+    const int slice = (int)(blockIdx.x % (unsigned)a.nslice);
+    const long long u0 = blockIdx.x / (unsigned)a.nslice, ustep = gridDim.x / (unsigned)a.nslice;
     const uint32_t ring_s = smem_u32(ring), w_s = smem_u32(wsm);
 
     if (warp == 0) {
@@ -203,7 +215,7 @@ __global__ void __launch_bounds__(ConvCfg<KC, N>::NTHREADS, 1)
             Ring<PLANES> r;
             long long issued = 0;
             bool stop = false;
-            for (long long u = blockIdx.x; u < nunits && !stop; u += gridDim.x) {
+            for (long long u = u0; u < nunits && !stop; u += ustep) {
                 const ConvUnit c = conv_unit(u, tx0, tiles_x, tiles_y, nzc, a.lz, a.D);
                 for (int p = c.z0 - 1; p <= c.z1; ++p) {
                     if (!mbar_wait_abort(smem_u32(&empty_b[r.s]), r.ph ^ 1, MBAR_LIMIT, &abort_s)) {
@@ -214,8 +226,8 @@ __global__ void __launch_bounds__(ConvCfg<KC, N>::NTHREADS, 1)
                     }
                     const uint32_t fb = smem_u32(&full_b[r.s]);
                     mbar_arrive_expect_tx(fb, Cfg::PLANE);
-                    tma_load_5d(ring_s + (uint32_t)(r.s * Cfg::PLANE), &tmap, a.cin_off, c.tx * TXO - 1, c.ty * TY - 1,
-                                p, c.b, fb);
+                    tma_load_5d(ring_s + (uint32_t)(r.s * Cfg::PLANE), &tmap, a.cin_off, c.tx * TXO, c.ty * TY - 1,
+                                p, EXT && a.bmod ? c.b % a.bmod : c.b, fb);
                     ++issued;
                     r.next();
                 }
@@ -247,7 +259,7 @@ __global__ void __launch_bounds__(ConvCfg<KC, N>::NTHREADS, 1)
         }
         int ps[3] = {0, 0, 0}; // ring slots of planes p - 2, p - 1, p
         bool stop = false;
-        for (long long u = blockIdx.x; u < nunits && !stop; u += gridDim.x) {
+        for (long long u = u0; u < nunits && !stop; u += ustep) {
             const ConvUnit c = conv_unit(u, tx0, tiles_x, tiles_y, nzc, a.lz, a.D);
             int s0 = ar.s;     // accumulator of output plane max(p - 1, z0)
             for (int p = c.z0 - 1; p <= c.z1; ++p) {
@@ -343,32 +355,37 @@ __global__ void __launch_bounds__(ConvCfg<KC, N>::NTHREADS, 1)
     } else {
         // ------------------------------------------------------------ epilogue
         const int q = warp & 3;                    // TMEM lane quarter this warp may access
-        const int grp = ((warp - 2) >> 2) % Cfg::NG;  // its 16 output channels
+        const int grp = ((warp - 2) >> 2) % Cfg::NG;  // its 16 output channels of the slice
         const int set = ((warp - 2) >> 2) / Cfg::NG;  // its share of the output planes
         const int m = q * 32 + lane;               // accumulator row = cell of the block
         const float scale = a.scale_out ? a.drop_scale : 1.0f;
         const uint64_t scale2 = f32x2(scale, scale);
         const int bx = m & (TX - 1);               // cell of the block row (0 and TX - 1 are halo)
         const long long opitch = a.out_pitch ? a.out_pitch : N;
-        const long long HW = (long long)a.H * a.W;
+        const long long HW = (long long)a.H * a.W, ostep = HW * opitch;
         // dropout threshold in both halves; its top bits pick the compare below
         const uint32_t thr = a.drop_thr, thr7 = (thr & 0x7FFFu) * 0x10001u, thr_low = thr < 0x8000u ? 0xFFFFFFFFu : 0u;
-        uint64_t bias[EPC / 2];
-#pragma unroll
-        for (int j = 0; j < EPC / 2; ++j)
-            bias[j] = a.bias ? f32x2(__ldg(a.bias + grp * EPC + 2 * j), __ldg(a.bias + grp * EPC + 2 * j + 1)) : 0ULL;
+        const int ch0 = a.out_off + slice * N + grp * EPC;  // first channel of the warp in the output
+        const uint32_t bias4 = smem_u32(bias_s + grp * EPC);
         Ring<NACC> ar;
         int turn = 0;
         bool stop = false;
-        for (long long u = blockIdx.x; u < nunits && !stop; u += gridDim.x) {
+        for (long long u = u0; u < nunits && !stop; u += ustep) {
             const ConvUnit c = conv_unit(u, tx0, tiles_x, tiles_y, nzc, a.lz, a.D);
-            const int cx = c.tx * TXO + bx - 1, cy = c.ty * TY + (m >> 4);
-            // the halo cells of the block row, and cells past the volume, write nothing
-            const bool valid = bx != 0 && bx != TX - 1 && cx < a.W;
+            const int cx = c.tx * TXO + bx, cy = c.ty * TY + (m >> 4);
+            // a block's first and last cell yield an output only where the volume ends there;
+            // cells past the volume write nothing
+            const bool valid = cx < a.W && (bx != 0 || cx == 0) && (bx != TX - 1 || cx == a.W - 1);
             uint32_t lin = (uint32_t)(((long long)c.z0 * a.H + cy) * a.W + (valid ? cx : 0));
-            long long obase = ((((long long)c.b * a.D + c.z0) * a.H + cy) * a.W + (valid ? cx : 0)) * opitch +
-                              a.out_off + grp * EPC;
-            for (int z = c.z0; z < c.z1; ++z, lin += (uint32_t)HW, obase += HW * opitch, ar.next()) {
+            long long obase = ((((long long)c.b * a.D + c.z0) * a.H + cy) * a.W + (valid ? cx : 0)) * opitch + ch0;
+            // where the shortcut of the cell lies
+            long long rbase = EXT ? ((((long long)(a.bmod ? c.b % a.bmod : c.b) * a.D + c.z0) * a.H + cy) * a.W +
+                                     (valid ? cx : 0)) * a.res_ch + ch0
+                                  : 0;
+            // several MC passes of one batch run side by side: sample b is pass b / pass_b's
+            const uint32_t bdrop = EXT && a.pass_b ? (uint32_t)c.b % (uint32_t)a.pass_b : (uint32_t)c.b;
+            const uint32_t pass = a.pass + (EXT && a.pass_b ? (uint32_t)c.b / (uint32_t)a.pass_b : 0u);
+            for (int z = c.z0; z < c.z1; ++z, lin += (uint32_t)HW, obase += ostep, ar.next()) {
                 const bool mine = turn == set;
                 if (++turn == Cfg::NSET) turn = 0;
                 if (!mine) continue;
@@ -380,8 +397,7 @@ __global__ void __launch_bounds__(ConvCfg<KC, N>::NTHREADS, 1)
                 if (thr) {
 #pragma unroll
                     for (int h = 0; h < EPC / 8; ++h) {
-                        const u32x4 r = philox4x32_10(lin, (uint32_t)c.b, (a.layer << 16) | (uint32_t)(grp * (EPC / 8) + h),
-                                                      a.pass, a.seed, 0xD0u);
+                        const u32x4 r = philox4x32_10(lin, bdrop, (a.layer << 16) | (uint32_t)(ch0 / 8 + h), pass, a.seed, 0xD0u);
 #pragma unroll
                         for (int w = 0; w < 4; ++w) {
                             // per half: bit 15 of t is (low 15 bits >= the threshold's)
@@ -411,61 +427,86 @@ __global__ void __launch_bounds__(ConvCfg<KC, N>::NTHREADS, 1)
                     fence_before_sync();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(smem_u32(&tempty_b[ar.s]));
-                    // lanes m - 1 and m + 1 are the x-neighbours (same block row for
-                    // the interior cells that produce output)
+                    // lanes m - 1 and m + 1 are the x-neighbours; the block row's first and last
+                    // cell have none where the volume ends there (elsewhere they write nothing)
 #pragma unroll
                     for (int o = 0; o < EPC; o += 2) {
-                        const uint64_t left = f32x2(__shfl_up_sync(0xffffffffu, p[o], 1),
-                                                    __shfl_up_sync(0xffffffffu, p[o + 1], 1));
-                        const uint64_t right = f32x2(__shfl_down_sync(0xffffffffu, p[2 * EPC + o], 1),
-                                                     __shfl_down_sync(0xffffffffu, p[2 * EPC + o + 1], 1));
+                        const float l0 = __shfl_up_sync(0xffffffffu, p[o], 1);
+                        const float l1 = __shfl_up_sync(0xffffffffu, p[o + 1], 1);
+                        const float r0 = __shfl_down_sync(0xffffffffu, p[2 * EPC + o], 1);
+                        const float r1 = __shfl_down_sync(0xffffffffu, p[2 * EPC + o + 1], 1);
+                        const uint64_t left = f32x2(bx == 0 ? 0.0f : l0, bx == 0 ? 0.0f : l1);
+                        const uint64_t right = f32x2(bx == TX - 1 ? 0.0f : r0, bx == TX - 1 ? 0.0f : r1);
                         v2[o / 2] = add2(add2(left, f32x2(p[EPC + o], p[EPC + o + 1])), right);
                     }
                 }
-                if (!valid) continue;
-                float v[EPC];
-                if (a.y_f32 && a.accum) {
+                if (valid) {
+                    if (EXT && a.part_in) {
+                        // the sums of the input-channel chunks before this one
+                        const float4 *p4 = reinterpret_cast<const float4 *>(a.part_in + obase);
 #pragma unroll
-                    for (int j = 0; j < EPC; j += 2) {
-                        const float2 s2 = unpack2(v2[j / 2]);
-                        v[j] = s2.x;
-                        v[j + 1] = s2.y;
+                        for (int j = 0; j < EPC / 4; ++j) {
+                            const float4 p0 = p4[j];
+                            v2[2 * j] = add2(f32x2(p0.x, p0.y), v2[2 * j]);
+                            v2[2 * j + 1] = add2(f32x2(p0.z, p0.w), v2[2 * j + 1]);
+                        }
                     }
-                    // partial sums of one input-channel chunk: add the raw accumulator
-                    float4 *o4 = reinterpret_cast<float4 *>(a.y_f32 + obase);
+                    if (EXT && a.raw_out) {
+                        float4 *o4 = reinterpret_cast<float4 *>(a.raw_out + obase);
 #pragma unroll
-                    for (int j = 0; j < EPC / 4; ++j) {
-                        const float4 p0 = o4[j];
-                        o4[j] = make_float4(p0.x + v[4 * j], p0.y + v[4 * j + 1], p0.z + v[4 * j + 2], p0.w + v[4 * j + 3]);
+                        for (int j = 0; j < EPC / 4; ++j) {
+                            const float2 s0 = unpack2(v2[2 * j]), s1 = unpack2(v2[2 * j + 1]);
+                            o4[j] = make_float4(s0.x, s0.y, s1.x, s1.y);
+                        }
                     }
-                    continue;
+                    float v[EPC];
+#pragma unroll
+                    for (int j = 0; j < EPC; j += 4) {
+                        // the bias stays in shared memory: the loop has no registers for it, and a
+                        // spill costs an L2 round trip here (the L1 is all shared memory)
+                        uint64_t b2[2];
+                        asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(b2[0]), "=l"(b2[1]) : "r"(bias4 + 4u * j));
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            float2 s2 = unpack2(add2(v2[j / 2 + h], b2[h]));
+                            if (a.relu) s2 = make_float2(fmaxf(s2.x, 0.0f), fmaxf(s2.y, 0.0f));
+                            s2 = unpack2(mul2(f32x2(s2.x, s2.y), scale2));
+                            v[j + 2 * h] = s2.x;
+                            v[j + 2 * h + 1] = s2.y;
+                        }
+                    }
+                    if (a.y_f32) {
+                        float4 *o4 = reinterpret_cast<float4 *>(a.y_f32 + obase);
+#pragma unroll
+                        for (int j = 0; j < EPC; ++j)
+                            if (!((keep[j >> 1] >> (16 * (j & 1))) & 1u)) v[j] = 0.0f;
+#pragma unroll
+                        for (int j = 0; j < EPC / 4; ++j)
+                            o4[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                    } else if (!EXT || a.y) {
+                        uint32_t o[EPC / 2];
+#pragma unroll
+                        for (int j = 0; j < EPC / 2; ++j) {
+                            const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+                            o[j] = *reinterpret_cast<const uint32_t *>(&h) & keep[j];
+                        }
+                        if (EXT && ch0 < a.res_ch) {
+                            // identity shortcut: the dropped-out FP32 value plus the layer's input, one rounding
+                            const uint4 *r4 = reinterpret_cast<const uint4 *>(a.res + rbase + (z - c.z0) * HW * a.res_ch);
+                            const uint4 ra = r4[0], rb = r4[1];
+                            const uint32_t rw[EPC / 2] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
+#pragma unroll
+                            for (int j = 0; j < EPC / 2; ++j) {
+                                const float x0 = __uint_as_float(rw[j] << 16), x1 = __uint_as_float(rw[j] & 0xFFFF0000u);
+                                const __nv_bfloat162 h = __floats2bfloat162_rn((keep[j] & 1u ? v[2 * j] : 0.0f) + x0,
+                                                                               (keep[j] >> 16 ? v[2 * j + 1] : 0.0f) + x1);
+                                o[j] = *reinterpret_cast<const uint32_t *>(&h);
+                            }
+                        }
+                        uint4 *o4 = reinterpret_cast<uint4 *>(a.y + obase);
+                        o4[0] = make_uint4(o[0], o[1], o[2], o[3]);
+                        o4[1] = make_uint4(o[4], o[5], o[6], o[7]);
                 }
-#pragma unroll
-                for (int j = 0; j < EPC; j += 2) {
-                    float2 s2 = unpack2(add2(v2[j / 2], bias[j / 2]));
-                    if (a.relu) s2 = make_float2(fmaxf(s2.x, 0.0f), fmaxf(s2.y, 0.0f));
-                    s2 = unpack2(mul2(f32x2(s2.x, s2.y), scale2));
-                    v[j] = s2.x;
-                    v[j + 1] = s2.y;
-                }
-                if (a.y_f32) {
-                    float4 *o4 = reinterpret_cast<float4 *>(a.y_f32 + obase);
-#pragma unroll
-                    for (int j = 0; j < EPC; ++j)
-                        if (!((keep[j >> 1] >> (16 * (j & 1))) & 1u)) v[j] = 0.0f;
-#pragma unroll
-                    for (int j = 0; j < EPC / 4; ++j)
-                        o4[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-                } else {
-                    uint32_t o[EPC / 2];
-#pragma unroll
-                    for (int j = 0; j < EPC / 2; ++j) {
-                        const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
-                        o[j] = *reinterpret_cast<const uint32_t *>(&h) & keep[j];
-                    }
-                    uint4 *o4 = reinterpret_cast<uint4 *>(a.y + obase);
-                    o4[0] = make_uint4(o[0], o[1], o[2], o[3]);
-                    o4[1] = make_uint4(o[4], o[5], o[6], o[7]);
                 }
             }
         }
@@ -502,7 +543,7 @@ static hyb_status make_tmap(CUtensorMap *tm, const ConvArgs &a) {
     EncodeTiledFn enc = encode_fn();
     if (!enc) return set_error(HYB_ECUDA, "cuTensorMapEncodeTiled is not available");
     const cuuint64_t C = (cuuint64_t)(a.cin_total ? a.cin_total : a.cin);
-    const cuuint64_t dims[5] = {C, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)a.D, (cuuint64_t)a.B};
+    const cuuint64_t dims[5] = {C, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)a.D, (cuuint64_t)(a.bmod ? a.bmod : a.B)};
     const cuuint64_t es = 2;
     const cuuint64_t strides[4] = {es * C, es * C * a.W, es * C * a.W * a.H, es * C * a.W * a.H * a.D};
     const cuuint32_t box[5] = {(cuuint32_t)a.cin, (cuuint32_t)TX, (cuuint32_t)HY, 1, 1};
@@ -514,7 +555,7 @@ static hyb_status make_tmap(CUtensorMap *tm, const ConvArgs &a) {
     return HYB_OK;
 }
 
-template <int KC, int N>
+template <int KC, int N, bool EXT>
 static hyb_status launch_cfg(const ConvArgs &a, cudaStream_t st) {
     using Cfg = ConvCfg<KC, N>;
     CUtensorMap tm;
@@ -530,7 +571,7 @@ static hyb_status launch_cfg(const ConvArgs &a, cudaStream_t st) {
     {
         std::lock_guard<std::mutex> lock(mu);
         if (!ready_dev[dev]) {
-            cudaError_t e = cudaFuncSetAttribute(k_conv3_tc<KC, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            cudaError_t e = cudaFuncSetAttribute(k_conv3_tc<KC, N, EXT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  Cfg::SMEM);
             if (e != cudaSuccess)
                 return set_error(HYB_ECUDA, std::string("conv smem attribute: ") + cudaGetErrorString(e));
@@ -548,18 +589,20 @@ static hyb_status launch_cfg(const ConvArgs &a, cudaStream_t st) {
     const long long cols = (long long)a.B * (a.H / TY) * ntx;
     if (cols == 0) return HYB_OK;
     ConvArgs b = a;
+    if (b.nslice < 1) b.nslice = 1;
+    const long long per = std::max(1, nsm / b.nslice);  // CTAs per output slice
     double best = 0.0;
     for (int lz = 2; lz <= 32; ++lz) {
         const long long u = cols * ((a.D + lz - 1) / lz);
-        const double t = (double)((u + nsm - 1) / nsm) * (std::min(lz, a.D) + 0.4);
+        const double t = (double)((u + per - 1) / per) * (std::min(lz, a.D) + 0.4);
         if (lz == 2 || t < best) {
             best = t;
             b.lz = lz;
         }
     }
     const long long units = cols * ((a.D + b.lz - 1) / b.lz);
-    const long long grid = std::min<long long>(units, (long long)nsm);  // one CTA per SM (all of its TMEM)
-    k_conv3_tc<KC, N><<<(unsigned)grid, Cfg::NTHREADS, Cfg::SMEM, st>>>(tm, b);
+    const long long grid = std::min<long long>(units, per) * b.nslice;  // one CTA per SM (all of its TMEM)
+    k_conv3_tc<KC, N, EXT><<<(unsigned)grid, Cfg::NTHREADS, Cfg::SMEM, st>>>(tm, b);
     e = cudaGetLastError();
     if (e != cudaSuccess) return set_error(HYB_ECUDA, std::string("conv launch: ") + cudaGetErrorString(e));
     return HYB_OK;
@@ -571,20 +614,23 @@ hyb_status launch_conv3_tc(const ConvArgs &a, cudaStream_t st) {
     if ((long long)a.B * a.D * (a.H / TY) * ((a.W + TXO - 1) / TXO) >= (1LL << 31))
         return set_error(HYB_EINVAL, "conv shape: more than 2^31 tiles");
     if (((uintptr_t)a.x & 15) || ((uintptr_t)a.y & 15) || ((uintptr_t)a.y_f32 & 15) || ((uintptr_t)a.wt & 15) ||
-        (!a.y && !a.y_f32))
+        ((uintptr_t)a.part_in & 15) || ((uintptr_t)a.raw_out & 15) || ((uintptr_t)a.res & 15) ||
+        (!a.y && !a.y_f32 && !a.raw_out))
         return set_error(HYB_EINVAL, "conv operands must be present and 16-byte aligned");
     {
-        // channel chunks: 16-channel aligned input slices (TMA x coordinate in
-        // 32-byte steps), 8-channel aligned output slices (16-byte stores)
+        // channel chunks: 16-channel aligned input and output slices (TMA x coordinate in
+        // 32-byte steps, 32-byte stores)
         const int ct = a.cin_total ? a.cin_total : a.cin, op = a.out_pitch ? a.out_pitch : a.N;
-        if (ct % 16 || a.cin_off < 0 || a.cin_off % 16 || a.cin_off + a.cin > ct || op % 8 || a.out_off < 0 ||
-            a.out_off % 8 || a.out_off + a.N > op || (a.accum && !a.y_f32))
+        const int ns = a.nslice > 1 ? a.nslice : 1;
+        if (ct % 16 || a.cin_off < 0 || a.cin_off % 16 || a.cin_off + a.cin > ct || op % 16 || a.out_off < 0 ||
+            a.out_off % 16 || a.out_off + ns * a.N > op || a.res_ch % 16 || (a.res_ch && !a.res))
             return set_error(HYB_EINVAL, "conv channel slices out of range or misaligned");
     }
-    if (a.cin == 16 && a.N == 32) return launch_cfg<2, 32>(a, st);
-    if (a.cin == 32 && a.N == 32) return launch_cfg<4, 32>(a, st);
-    if (a.cin == 32 && a.N == 16) return launch_cfg<4, 16>(a, st);
-    if (a.cin == 16 && a.N == 16) return launch_cfg<2, 16>(a, st);
+    const bool ext = a.part_in || a.raw_out || a.res_ch || a.bmod || a.pass_b;
+    if (a.cin == 16 && a.N == 32) return ext ? launch_cfg<2, 32, true>(a, st) : launch_cfg<2, 32, false>(a, st);
+    if (a.cin == 32 && a.N == 32) return ext ? launch_cfg<4, 32, true>(a, st) : launch_cfg<4, 32, false>(a, st);
+    if (a.cin == 32 && a.N == 16) return ext ? launch_cfg<4, 16, true>(a, st) : launch_cfg<4, 16, false>(a, st);
+    if (a.cin == 16 && a.N == 16) return ext ? launch_cfg<2, 16, true>(a, st) : launch_cfg<2, 16, false>(a, st);
     return set_error(HYB_EINVAL, "conv channels: (C_in, C_out) in {16, 32} x {16, 32}");
 }
 

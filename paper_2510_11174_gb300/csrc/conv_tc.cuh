@@ -319,24 +319,33 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float v[16]) {
 
 namespace hyb {
 
-// one 3x3x3 convolution layer on the tensor cores (see conv.cu)
+// one 3x3x3 convolution layer on the tensor cores (see conv.cu).  With s the
+// sum over the launch's input channels (plus part_in), a launch writes any of
+//   raw_out = s                                         FP32
+//   y / y_f32 = drop(relu(s + bias)) scale [+ res]      BF16 / FP32 (FP32 without res)
 struct ConvArgs {
     const __nv_bfloat16 *x;   // [B][D][H][W][cin] channels-last
-    const __nv_bfloat16 *wt;  // [27][cin/8][N][8] core layout
-    const float *bias;        // [N] or null
+    const __nv_bfloat16 *wt;  // [nslice][27][cin/8][N][8] core layout
+    const float *bias;        // [out_pitch] or null
     __nv_bfloat16 *y;         // [B][D][H][W][N]
-    float *y_f32;             // when set: FP32 output [B][D][H][W][N] instead of y
+    float *y_f32;             // FP32 output [B][D][H][W][N] instead of y
+    const float *part_in;     // sums of earlier input-channel chunks [cells][out_pitch], or null
+    float *raw_out;           // sums so far [cells][out_pitch], or null
+    const __nv_bfloat16 *res; // identity shortcut [cells][res_ch]: added to the channels below res_ch (0: none)
+    int res_ch;
     int B, D, H, W, cin, N;   // cin: the channels one launch contracts (16 or 32)
+    int bmod;                 // the input (and res) holds bmod samples, sample b reads b % bmod (0: B samples)
     int cin_total;            // channel pitch of x (0: cin); a launch reads channels cin_off .. cin_off + cin - 1
     int cin_off;
-    int out_pitch;            // channel pitch of y / y_f32 (0: N); a launch writes channels out_off .. out_off + N - 1
-    int out_off;
-    int accum;                // y_f32 += the raw sums (no bias, ReLU or dropout): the partial of one input chunk
+    int out_pitch;            // channel pitch of the outputs (0: N); a launch writes channels
+    int out_off;              // out_off .. out_off + nslice N - 1
+    int nslice;               // output slices of N channels (0: 1)
     int relu;
     uint32_t drop_thr;        // dropout threshold round(p 2^16) on 16-bit Philox fields; 0: no dropout
     float drop_scale;         // 1 / (1 - drop_thr 2^-16)
     int scale_out;            // kept outputs are multiplied by drop_scale (set with dropout; alone: scaling only)
     uint32_t seed, pass, layer;
+    int pass_b;               // samples per pass: sample b takes the mask of sample b % pass_b of pass + b / pass_b (0: one pass)
     int *status;
     int x_lo, x_hi;           // when x_hi > x_lo: only the tiles whose outputs meet x_lo <= x < x_hi
     int lz;                   // output planes per column of blocks (set by the launch)

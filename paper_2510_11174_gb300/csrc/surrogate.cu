@@ -4,11 +4,11 @@
 // of a patch, trained with a Huber loss and a penalty on energy violation).
 //
 // The six 3x3x3 convolutions run on the classifier's tcgen05 kernel
-// (k_conv3_tc) in channel chunks: one launch contracts 16 or 32 input
-// channels into 16 or 32 output channels and adds its raw sums into the
-// layer's FP32 pre-activation buffer (k_conv3_tc's accumulate mode); a
-// finishing kernel adds the bias, applies ReLU, dropout and the identity
-// shortcut, and stores the BF16 activation.  The data gradient is the same
+// (k_conv3_tc): one launch contracts 16 or 32 input channels into all output
+// channels (its CTAs share the 16- or 32-channel output slices); a layer with
+// more input channels passes FP32 sums from launch to launch, and the last one's
+// epilogue adds the bias, applies ReLU, dropout and the identity shortcut, and
+// stores the BF16 activation.  The data gradient is the same
 // convolution with the transposed, flipped kernel; the weight gradient is the
 // tensor-core contraction over the cells (wgrad_tc);
 // Adam updates FP32 masters.  See hyb_surrogate_* in include/hyb.h.
@@ -104,6 +104,7 @@ constexpr int CIP[SL] = {16, 16, 32, 64, 128, 32}, COP[SL] = {16, 32, 64, 128, 3
 constexpr int RES[SL] = {1, 1, 1, 0, 0, 0};                      // identity shortcut (zero-padded channels)
 constexpr int RELU[SL] = {1, 1, 1, 1, 1, 0};
 constexpr int DROP_LAYER = 1;                                    // dropout after layer 1's ReLU
+constexpr long long MC_CELLS = 262144;                           // cells of the MC passes run side by side
 constexpr int NCH = 10;                                          // state channels: E, B, J, rho
 constexpr int RB = 256;
 
@@ -133,22 +134,27 @@ __global__ void k_sur_out(const float *__restrict__ y, const float *__restrict__
     out[t] = x[t] + y[(b * V + v) * 16 + c] * sd[c];
 }
 
-// MC statistics: pass k (1-based) folded into the running mean and M2 (Welford)
+// MC statistics: passes k .. k + g - 1 (1-based; y holds them one after the other)
+// folded in order into the running mean and M2 (Welford)
 __global__ void k_sur_mc(const float *__restrict__ y, const float *__restrict__ x, int B, long long V,
-                         const float *__restrict__ sd, int k, float *__restrict__ pm, float *__restrict__ m2) {
+                         const float *__restrict__ sd, int k, int g, float *__restrict__ pm, float *__restrict__ m2) {
     const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (t >= (long long)B * V * NCH) return;
     const long long b = t / (V * NCH), c = (t / V) % NCH, v = t % V;
-    const float val = x[t] + y[(b * V + v) * 16 + c] * sd[c];
-    if (k == 1) {
-        pm[t] = val;
-        m2[t] = 0.0f;
-    } else {
-        const float d = val - pm[t];
-        const float mu = pm[t] + d / (float)k;
-        pm[t] = mu;
-        m2[t] += d * (val - mu);
+    float mean = k == 1 ? 0.0f : pm[t], q = k == 1 ? 0.0f : m2[t];
+    for (int i = 0; i < g; ++i) {
+        const float val = x[t] + y[((i * B + b) * V + v) * 16 + c] * sd[c];
+        if (k + i == 1) {
+            mean = val;
+        } else {
+            const float d = val - mean;
+            const float mu = mean + d / (float)(k + i);
+            mean = mu;
+            q += d * (val - mu);
+        }
     }
+    pm[t] = mean;
+    m2[t] = q;
 }
 
 __global__ void k_sur_mc_final(long long n, int k, float *__restrict__ m2) {
@@ -382,33 +388,35 @@ hyb_status reserve(hyb_surrogate *m, long long cells) {
     return HYB_OK;
 }
 
-// acc [cells][nout] (zeroed) += conv(x [cells][nin]; the packs pk) in channel chunks
+// conv(x [cells][nin]; the packs pk) -> nout channels: one launch per input-channel
+// chunk, which sums into FP32 `sums` [cells][nout] up to the last; that one
+// writes `fin` (its outputs and epilogue), and the sums too when keep_sums
 hyb_status conv_chunks(hyb_surrogate *m, const __nv_bfloat16 *x, int nin, const __nv_bfloat16 *pk, int nout,
-                       float *acc, int B, int D, int H, int W) {
-    const int cic = chunk_of(nin), nsl = chunk_of(nout), nos = nout / nsl;
+                       float *sums, bool keep_sums, const ConvArgs &fin, int B, int D, int H, int W) {
+    const int cic = chunk_of(nin), nsl = chunk_of(nout), nos = nout / nsl, nic = nin / cic;
     const long long blk = 27LL * cic * nsl;
-    for (int ic = 0; ic < nin / cic; ++ic)
-        for (int os = 0; os < nos; ++os) {
-            ConvArgs a;
-            memset(&a, 0, sizeof(a));
-            a.x = x;
-            a.wt = pk + (ic * nos + os) * blk;
-            a.B = B;
-            a.D = D;
-            a.H = H;
-            a.W = W;
-            a.cin = cic;
-            a.cin_total = nin;
-            a.cin_off = ic * cic;
-            a.N = nsl;
-            a.y_f32 = acc;
-            a.out_pitch = nout;
-            a.out_off = os * nsl;
-            a.accum = 1;
-            a.status = m->status;
-            hyb_status st = launch_conv3_tc(a, m->stream);
-            if (st != HYB_OK) return st;
-        }
+    for (int ic = 0; ic < nic; ++ic) {
+        ConvArgs a;
+        if (ic == nic - 1) a = fin;
+        else memset(&a, 0, sizeof(a));
+        a.x = x;
+        a.wt = pk + ic * nos * blk;
+        a.B = B;
+        a.D = D;
+        a.H = H;
+        a.W = W;
+        a.cin = cic;
+        a.cin_total = nin;
+        a.cin_off = ic * cic;
+        a.N = nsl;
+        a.nslice = nos;
+        a.out_pitch = nout;
+        a.part_in = ic > 0 ? sums : nullptr;
+        a.raw_out = ic < nic - 1 || keep_sums ? sums : nullptr;
+        a.status = m->status;
+        hyb_status st = launch_conv3_tc(a, m->stream);
+        if (st != HYB_OK) return st;
+    }
     return HYB_OK;
 }
 
@@ -425,20 +433,41 @@ DropArgs drop_of(const hyb_surrogate *m, int l, int pass) {
     return dr;
 }
 
-// forward pass of prepared inputs m->a[0] -> m->y
-hyb_status forward(hyb_surrogate *m, int B, int D, int H, int W, int pass) {
-    const long long V = (long long)D * H * W, cells = (long long)B * V;
-    for (int l = 0; l < SL; ++l) {
-        cudaMemsetAsync(m->s[l], 0, sizeof(float) * COP[l] * cells, m->stream);
-        hyb_status st = conv_chunks(m, m->a[l], CIP[l], m->pk[l], COP[l], m->s[l], B, D, H, W);
+// layers first .. last of the forward pass (m->a[first] -> m->a[last + 1], or m->y).
+// The convolution's own epilogue applies bias, ReLU, dropout and the shortcut;
+// `train` keeps the pre-activation sums s[l] the backward pass reads.  With
+// groups > 1, passes pass .. pass + groups - 1 of a batch of B samples run side
+// by side from the layer that drops out on (it reads the one input they share).
+hyb_status forward(hyb_surrogate *m, int first, int last, int B, int D, int H, int W, int pass, int groups, bool train) {
+    for (int l = first; l <= last; ++l) {
+        const bool shared = l < DROP_LAYER;
+        ConvArgs a;
+        memset(&a, 0, sizeof(a));
+        a.bias = m->b[l];
+        a.relu = RELU[l];
+        if (l == SL - 1) a.y_f32 = m->y;
+        else a.y = m->a[l + 1];
+        if (RES[l]) {
+            a.res = m->a[l];
+            a.res_ch = CIP[l];
+        }
+        if (l == DROP_LAYER) {
+            a.bmod = B;
+            if (pass >= 0) {
+                const uint32_t thr = dropout_threshold(m->d.dropout);
+                a.drop_thr = thr;
+                a.drop_scale = dropout_scale(thr);
+                a.scale_out = thr != 0;
+                a.seed = m->d.seed;
+                a.pass = (uint32_t)pass;
+                a.layer = (uint32_t)l;
+                a.pass_b = B;
+            }
+        }
+        const hyb_status st = conv_chunks(m, m->a[l], CIP[l], m->pk[l], COP[l], m->s[l], train && l < SL - 1, a,
+                                          shared ? B : B * groups, D, H, W);
         if (st != HYB_OK) return st;
-        const bool last = l == SL - 1;
-        k_act_finish<<<nbk(cells * (COP[l] / 8)), RB, 0, m->stream>>>(
-            m->s[l], m->b[l], COP[l], RELU[l], RES[l] ? m->a[l] : nullptr, CIP[l], drop_of(m, l, pass), B, V,
-            last ? nullptr : m->a[l + 1], last ? m->y : nullptr);
     }
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return set_error(HYB_ECUDA, std::string("surrogate forward: ") + cudaGetErrorString(e));
     return HYB_OK;
 }
 
@@ -598,7 +627,7 @@ hyb_status hyb_surrogate_forward(hyb_surrogate *m, const float *x, int B, int D,
     if (s == HYB_OK) s = reserve(m, cells);
     if (s != HYB_OK) return s;
     k_sur_prep<<<nbk(cells), RB, 0, m->stream>>>(x, B, V, m->mean, m->std_, m->a[0]);
-    if ((s = forward(m, B, D, H, W, pass)) != HYB_OK) return s;
+    if ((s = forward(m, 0, SL - 1, B, D, H, W, pass, 1, false)) != HYB_OK) return s;
     k_sur_out<<<nbk(cells * NCH), RB, 0, m->stream>>>(m->y, x, B, V, m->dstd, y);
     HYB_CUDA_TRY(cudaGetLastError());
     return HYB_OK;
@@ -608,13 +637,18 @@ hyb_status hyb_surrogate_mc(hyb_surrogate *m, const float *x, int B, int D, int 
     if (!m || !x || !pm || !ps) return set_error(HYB_EINVAL, "null argument");
     hyb_status s = check_shape(B, D, H, W);
     const long long V = (long long)D * H * W, cells = (long long)B * V;
-    if (s == HYB_OK) s = reserve(m, cells);
+    // as many passes side by side as keep a launch's volume within MC_CELLS: a small
+    // batch does not fill the SMs (65 536 cells: four passes, 6.3 -> 1.9 ms for 16)
+    const int K = m->d.mc_passes;
+    const int G = (int)std::max<long long>(1, std::min<long long>(K, MC_CELLS / cells));
+    if (s == HYB_OK) s = reserve(m, cells * G);
     if (s != HYB_OK) return s;
     k_sur_prep<<<nbk(cells), RB, 0, m->stream>>>(x, B, V, m->mean, m->std_, m->a[0]);
-    const int K = m->d.mc_passes;
-    for (int k = 1; k <= K; ++k) {
-        if ((s = forward(m, B, D, H, W, k - 1)) != HYB_OK) return s;
-        k_sur_mc<<<nbk(cells * NCH), RB, 0, m->stream>>>(m->y, x, B, V, m->dstd, k, pm, ps);
+    if ((s = forward(m, 0, DROP_LAYER - 1, B, D, H, W, -1, 1, false)) != HYB_OK) return s;
+    for (int k = 0; k < K; k += G) {
+        const int g = std::min(G, K - k);
+        if ((s = forward(m, DROP_LAYER, SL - 1, B, D, H, W, k, g, false)) != HYB_OK) return s;
+        k_sur_mc<<<nbk(cells * NCH), RB, 0, m->stream>>>(m->y, x, B, V, m->dstd, k + 1, g, pm, ps);
     }
     k_sur_mc_final<<<nbk(cells * NCH), RB, 0, m->stream>>>(cells * NCH, K, ps);
     HYB_CUDA_TRY(cudaGetLastError());
@@ -641,7 +675,7 @@ hyb_status hyb_surrogate_train_step(hyb_surrogate *m, const float *x, const floa
     cudaStream_t st = m->stream;
     const int pass = (int)(m->adam_t & 0x7fffffff);
     k_sur_prep<<<nbk(cells), RB, 0, st>>>(x, B, V, m->mean, m->std_, m->a[0]);
-    if ((s = forward(m, B, D, H, W, pass)) != HYB_OK) return s;
+    if ((s = forward(m, 0, SL - 1, B, D, H, W, pass, 1, true)) != HYB_OK) return s;
     // loss: per-sample energies, then the gradient dL/dy (G[SL] and dz)
     k_sur_energy<<<dim3(m->eblocks, B), RB, 0, st>>>(m->y, tg, x, V, m->dstd, m->epart);
     k_sur_esum<<<nbk(B), RB, 0, st>>>(m->epart, B, m->eblocks, m->esum);
@@ -654,8 +688,9 @@ hyb_status hyb_surrogate_train_step(hyb_surrogate *m, const float *x, const floa
                                                               drop_of(m, l, pass), B, V, m->dz);
         if ((s = layer_wgrad(m, l, B, D, H, W)) != HYB_OK) return s;
         if (l > 0) {
-            cudaMemsetAsync(m->G[l], 0, sizeof(float) * CIP[l] * cells, st);
-            if ((s = conv_chunks(m, m->dz, COP[l], m->pkT[l], CIP[l], m->G[l], B, D, H, W)) != HYB_OK) return s;
+            ConvArgs a;
+            memset(&a, 0, sizeof(a));
+            if ((s = conv_chunks(m, m->dz, COP[l], m->pkT[l], CIP[l], m->G[l], true, a, B, D, H, W)) != HYB_OK) return s;
             if (RES[l]) k_sur_addres<<<nbk(cells * CIP[l]), RB, 0, st>>>(m->G[l], m->G[l + 1], CIP[l], COP[l], cells);
         }
     }
