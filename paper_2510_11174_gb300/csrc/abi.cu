@@ -78,7 +78,6 @@ static void enqueue_step(hyb_ctx *c) {
     const SpSet set = species_set(c);
     PhaseMark pm{c};
     for (int p = 0; p < HYB_PH_CLASSIFY; ++p) c->phase_ran[p] = false;
-    cudaMemsetAsync(c->mig_counts, 0, sizeof(int) * HYB_MAX_SPECIES, st);
     if (set.n > 0) {
         pm.begin(HYB_PH_PUSH);
         bool events = false;
@@ -106,10 +105,8 @@ static void enqueue_step(hyb_ctx *c) {
     }
     if (set.n > 0) {
         pm.begin(HYB_PH_REBIN);
-        for (int s = 0; s < set.n; ++s) {
-            launch_rebin(g, set.s[s], c->status, st);
-            launch_compact(g, set.s[s], st);
-        }
+        launch_rebin(c->sp_dev, set.n, c->status, st);
+        launch_compact(g, c->sp_dev, set.n, c->step_dev, st);  // also advances the step
         pm.end(HYB_PH_REBIN);
     }
     pm.begin(HYB_PH_FIELD);
@@ -118,14 +115,14 @@ static void enqueue_step(hyb_ctx *c) {
     launch_mur(g, c->E, c->mur_old, c->mur_plane, st);
     launch_fdtd_b_half(g, c->E, c->B, st);
     pm.end(HYB_PH_FIELD);
-    launch_step_inc(c->step_dev, st);
+    if (set.n == 0) launch_step_inc(c->step_dev, st);
 
     // kernels enqueued above (memsets and event records are not kernels)
     long long k = 0;
-    if (set.n > 0) k += 2 + 2LL * set.n;
+    if (set.n > 0) k += 4;
     if (fluid_phase) k += 2;
     if (c->desc.laser_kind == HYB_LASER_GAUSS) k += 1;
-    k += 3 + ((g.bc[0] || g.bc[1] || g.bc[2]) ? 3 : 0) + 1;
+    k += 3 + ((g.bc[0] || g.bc[1] || g.bc[2]) ? 3 : 0) + (set.n == 0 ? 1 : 0);
     c->launches_per_step = k;
 }
 
@@ -293,6 +290,7 @@ hyb_status hyb_init_grid(const hyb_grid_desc *d, hyb_ctx **out) {
     cudaMemsetAsync(c->mur_old, 0, sizeof(float) * 24 * (size_t)c->mur_plane, st);
     cudaMemsetAsync(c->status, 0, sizeof(int), st);
     cudaMemsetAsync(c->step_dev, 0, sizeof(long long), st);
+    cudaMemsetAsync(c->mig_counts, 0, sizeof(int) * HYB_MAX_SPECIES, st);  // a step leaves them empty
     cudaMemsetAsync(c->mask, 0, (size_t)g.N, st);  // no node has switched to kinetic before a classification
     cudaMemsetAsync(c->fill_flags, 0, sizeof(int), st);
     cudaMemsetAsync(c->fluid_xr, 0, 2 * sizeof(int), st);  // every plane

@@ -367,8 +367,9 @@ hyb_status eval_qed(hyb_ctx *c, int what, const float *chi, const float *r, int 
 hyb_status setup_ionization(hyb_ctx *c, SpDev &s, const hyb_species_desc *d);
 hyb_status eval_ion_table(hyb_ctx *c, const SpDev &s, int Z, const float *x_host, int n, float *out_host);
 void launch_j_reduce(const GridDev &g, const float *jscratch, const int *jvalid, float *J, cudaStream_t st);
-void launch_rebin(const GridDev &g, const SpDev &s, int *status, cudaStream_t st);
-void launch_compact(const GridDev &g, const SpDev &s, cudaStream_t st);
+void launch_rebin(const SpDev *sps_dev, int nsp, int *status, cudaStream_t st);
+// step_dev (or null): advance the step counter and empty the migration buffers
+void launch_compact(const GridDev &g, const SpDev *sps_dev, int nsp, long long *step_dev, cudaStream_t st);
 void launch_regrid(const GridDev &g, const SpDev &from, const SpDev &to, cudaStream_t st);
 void launch_bin_particles(const GridDev &g, const SpDev &s, long long n, const float *x, const float *y,
                           const float *z, const float *ux, const float *uy, const float *uz, const float *w,

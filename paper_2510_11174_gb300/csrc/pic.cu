@@ -49,7 +49,7 @@ __host__ __device__ constexpr int push_threads(int T) { return T == 8 ? 256 : 12
 // CTAs per SM by shared memory (8^3: 73 KB linear, 114 KB quadratic shape; 4^3: 25 and 42 KB) and registers
 __host__ __device__ constexpr int push_ctas(int T, int order) { return T == 8 ? (order == 1 ? 3 : 2) : (order == 1 ? 6 : 5); }
 static constexpr int PUSH_Q = 32;          // entries of a per-warp queue of cell-crossing particles
-static constexpr int PUSH_SPLIT_CTAS = 512;   // see launch_push_deposit
+static constexpr int PUSH_SPLIT_CTAS = 456;   // see launch_push_deposit
 
 __host__ __device__ constexpr size_t align16(size_t b) { return (b + 15) & ~(size_t)15; }
 
@@ -434,6 +434,59 @@ __device__ __forceinline__ void queue_put(float4 *qa, int &n, bool want, const f
     }
 }
 
+// The stochastic events of the push, out of line: a step has few of them, and
+// their code (random numbers, table searches, the writes of new particles) in
+// the particle loop costs every warp instruction cache and registers (spills
+// 188 -> 132 bytes a thread, with the tallies straight to shared memory; a carbon
+// slab of 1.8 M particles with all three events, three runs side by side: five
+// steps 2024 -> 1905 us).
+static __device__ __noinline__ void event_spawn(const SpDev *d, float x, float y, float z, float ux, float uy, float uz,
+                                                float w, uint64_t id, int dest, long long step, uint32_t seed, float tau,
+                                                int *status) {
+    const float xs[3] = {x, y, z}, us[3] = {ux, uy, uz};
+    spawn(*d, xs, us, w, id, dest, step, seed, tau, status);
+}
+
+// Photon emission of particle `id` (species si; new position x, momentum u,
+// Lorentz factor gl).  Returns the factor on its momentum, its next optical
+// depth and the photon's energy where no photon particle is made (0 otherwise).
+static __device__ __noinline__ float3 event_emit(const SpDev *sps, int si, const QedDev *qd, float chi, float gl, float x,
+                                                 float y, float z, float ux, float uy, float uz, float w, uint64_t id,
+                                                 int dest, long long step, uint32_t seed, int *status) {
+    const SpDev &sp = sps[si];
+    const u32x4 r = philox4x32_10((uint32_t)id, (uint32_t)(id >> 32), (uint32_t)step, RNG_QED_EMIT, seed, sp.sp_index);
+    const float xi = qed_em_sample(*qd, chi, u01f(r.v[0]));
+    const float eps = fminf(xi * gl, gl - 1.0f);
+    const float g1 = gl - eps;
+    const float un = sqrtf(ux * ux + uy * uy + uz * uz);
+    const float u1 = sqrtf(fmaxf(g1 * g1 - 1.0f, 0.0f));
+    float lost = 0.0f;
+    if (eps >= sp.eps_min && sp.ph_species >= 0 && un > 0.0f)
+        event_spawn(&sps[sp.ph_species], x, y, z, eps * ux / un, eps * uy / un, eps * uz / un, w, derived_id(id, step, 2u),
+                    dest, step, seed, -logf(u01f(r.v[2])), status);
+    else lost = eps;
+    return make_float3(un > 0.0f ? u1 / un : 0.0f, -logf(u01f(r.v[1])), lost);
+}
+
+// Breit-Wheeler pair of photon `id` (momentum u, energy eps).  Returns the
+// energies of the two that fall short of a rest mass.
+static __device__ __noinline__ float2 event_pair(const SpDev *sps, int si, const QedDev *qd, float chi, float eps, float x,
+                                                 float y, float z, float ux, float uy, float uz, float w, uint64_t id,
+                                                 int dest, long long step, uint32_t seed, int *status) {
+    const SpDev &sp = sps[si];
+    const u32x4 r = philox4x32_10((uint32_t)id, (uint32_t)(id >> 32), (uint32_t)step, RNG_QED_PAIR, seed, sp.sp_index);
+    const float xi = qed_pair_sample(*qd, chi, u01f(r.v[0]));
+    const float en[2] = {xi * eps, (1.0f - xi) * eps};
+#pragma unroll 1
+    for (int k = 0; k < 2; ++k) {
+        const float p = en[k] > 1.0f ? sqrtf(en[k] * en[k] - 1.0f) : 0.0f;
+        event_spawn(&sps[k == 0 ? sp.pair_e : sp.pair_p], x, y, z, p * ux / eps, p * uy / eps, p * uz / eps, w,
+                    derived_id(id, step, k == 0 ? 3u : 5u), dest, step, seed, -logf(u01f(k == 0 ? r.v[1] : r.v[2])),
+                    status);
+    }
+    return make_float2(en[0] < 1.0f ? 1.0f - en[0] : 0.0f, en[1] < 1.0f ? 1.0f - en[1] : 0.0f);
+}
+
 // One CTA per tile (SPLIT: a cluster of CTAs per tile, each taking every
 // cluster-size-th block of its particles): stage E, B of the tile and a
 // one-node halo, push every particle of every species, deposit its current into
@@ -456,7 +509,7 @@ template <int T, int ORDER, bool EV, bool SPLIT>
 __global__ void __launch_bounds__(push_threads(T), push_ctas(T, ORDER))
     k_push_deposit(GridDev g, const float *__restrict__ E, const float *__restrict__ B,
                    const SpDev *__restrict__ sps, int nsp, float *__restrict__ jscratch, int *__restrict__ jvalid,
-                   int *__restrict__ status, const long long *__restrict__ step_dev, QedDev qd) {
+                   int *__restrict__ status, const long long *__restrict__ step_dev, const __grid_constant__ QedDev qd) {
     constexpr int F = frame_F(T, ORDER), G = frame_G(T, ORDER);
     constexpr int F3 = F * F * F, G3 = G * G * G;
     constexpr int NT = push_threads(T), NW = NT / 32;
@@ -584,8 +637,11 @@ __global__ void __launch_bounds__(push_threads(T), push_ctas(T, ORDER))
 
     for (int si = 0; si < nsp; ++si) {
         const SpDev &sp = s_sp[si];
-        double tal_e[NTALLY] = {0.0, 0.0, 0.0};
-        int tal_n[NTALLY] = {0, 0, 0};
+        // events are rare: their tallies go straight to shared memory, no registers held for them
+        auto tally = [&](int k, double energy) {
+            if (energy != 0.0) atomicAdd(&s_tal_e[si * NTALLY + k], energy);
+            atomicAdd(&s_tal_n[si * NTALLY + k], 1ULL);
+        };
         const int n = min(sp.count[t], sp.cap);
         const long long base = (long long)t * sp.cap;
         // times q_p below; photons (m = 0, q = 0) get no Lorentz force
@@ -747,11 +803,10 @@ __global__ void __launch_bounds__(push_threads(T), push_ctas(T, ORDER))
                                                   g.seed, sp.sp_index);
                     if (u01f(r.v[0]) < P) {
                         zq_new = (float)(Z + 1);
-                        tal_e[TALLY_IONIZE] += (double)wgt * sp.ip_mc2[Z];
-                        tal_n[TALLY_IONIZE] += 1;
-                        const SpDev &el = s_sp[sp.ion_into];
+                        tally(TALLY_IONIZE, (double)wgt * sp.ip_mc2[Z]);
                         const uint64_t eid = (1ULL << 63) | (pid << 3) | (uint64_t)(Z + 1);
-                        spawn(el, x1, u, wgt, eid, nt, step, g.seed, -1.0f, status);
+                        event_spawn(&s_sp[sp.ion_into], x1[0], x1[1], x1[2], u[0], u[1], u[2], wgt, eid, nt, step, g.seed,
+                                    -1.0f, status);
                     }
                 }
                 if (sp.qed) {
@@ -760,28 +815,12 @@ __global__ void __launch_bounds__(push_threads(T), push_ctas(T, ORDER))
                     const float chi = qed_chi(qd.kappa, e, b, u, gl);
                     tau -= qd.pref * qed_h(qd, chi) / gl * dt;
                     if (tau <= 0.0f) {
-                        const u32x4 r = philox4x32_10((uint32_t)pid, (uint32_t)(pid >> 32), (uint32_t)step,
-                                                      RNG_QED_EMIT, g.seed, sp.sp_index);
-                        const float xi = qed_em_sample(qd, chi, u01f(r.v[0]));
-                        tau = -logf(u01f(r.v[1]));
-                        const float eps = fminf(xi * gl, gl - 1.0f);
-                        const float g1 = gl - eps;
-                        const float un = sqrtf(u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
-                        const float u1 = sqrtf(fmaxf(g1 * g1 - 1.0f, 0.0f));
-                        const float sc = un > 0.0f ? u1 / un : 0.0f;
-                        float k[3];
+                        const float3 ev = event_emit(s_sp, si, &qd, chi, gl, x1[0], x1[1], x1[2], u[0], u[1], u[2], wgt,
+                                                     pid, nt, step, g.seed, status);
 #pragma unroll
-                        for (int c = 0; c < 3; ++c) {
-                            k[c] = un > 0.0f ? eps * u[c] / un : 0.0f;
-                            u[c] *= sc;
-                        }
-                        tal_n[TALLY_EMIT] += 1;
-                        if (eps >= sp.eps_min && sp.ph_species >= 0 && un > 0.0f) {
-                            spawn(s_sp[sp.ph_species], x1, k, wgt, derived_id(pid, step, 2u), nt, step, g.seed,
-                                  -logf(u01f(r.v[2])), status);
-                        } else {
-                            tal_e[TALLY_EMIT] += (double)wgt * eps;
-                        }
+                        for (int c = 0; c < 3; ++c) u[c] *= ev.x;
+                        tau = ev.y;
+                        tally(TALLY_EMIT, (double)wgt * ev.z);
                     }
                 }
                 if (sp.kind == 1 && sp.pair_e >= 0) {
@@ -791,25 +830,9 @@ __global__ void __launch_bounds__(push_threads(T), push_ctas(T, ORDER))
                         const float chi = qed_chi(qd.kappa, e, b, u, eps);
                         tau -= qd.pref * qed_T(qd, chi) / eps * dt;
                         if (tau <= 0.0f) {
-                            const u32x4 r = philox4x32_10((uint32_t)pid, (uint32_t)(pid >> 32), (uint32_t)step,
-                                                          RNG_QED_PAIR, g.seed, sp.sp_index);
-                            const float xi = qed_pair_sample(qd, chi, u01f(r.v[0]));
-                            const float ee = xi * eps, ep = (1.0f - xi) * eps;
-                            const float ue = ee > 1.0f ? sqrtf(ee * ee - 1.0f) : 0.0f;
-                            const float up = ep > 1.0f ? sqrtf(ep * ep - 1.0f) : 0.0f;
-                            if (ee < 1.0f) tal_e[TALLY_PAIR] += (double)wgt * (1.0f - ee);
-                            if (ep < 1.0f) tal_e[TALLY_PAIR] += (double)wgt * (1.0f - ep);
-                            tal_n[TALLY_PAIR] += 1;
-                            float ve[3], vp[3];
-#pragma unroll
-                            for (int c = 0; c < 3; ++c) {
-                                ve[c] = ue * u[c] / eps;
-                                vp[c] = up * u[c] / eps;
-                            }
-                            spawn(s_sp[sp.pair_e], x1, ve, wgt, derived_id(pid, step, 3u), nt, step, g.seed,
-                                  -logf(u01f(r.v[1])), status);
-                            spawn(s_sp[sp.pair_p], x1, vp, wgt, derived_id(pid, step, 5u), nt, step, g.seed,
-                                  -logf(u01f(r.v[2])), status);
+                            const float2 ev = event_pair(s_sp, si, &qd, chi, eps, x1[0], x1[1], x1[2], u[0], u[1],
+                                                         u[2], wgt, pid, nt, step, g.seed, status);
+                            tally(TALLY_PAIR, (double)wgt * ev.x + (double)wgt * ev.y);
                             dead = true;
                         }
                     }
@@ -866,23 +889,6 @@ __global__ void __launch_bounds__(push_threads(T), push_ctas(T, ORDER))
         }
         // the rest of the warp's last chunk holds no migrant
         if (lane >= mused && mbase + lane < sp.mig_cap) sp.mdest[mbase + lane] = -1;
-        if constexpr (EV) {
-            // per-tile tallies: warp sums, then shared accumulators, then one add per tile
-            if (sp.zmax > 0 || sp.qed || sp.pair_e >= 0) {
-#pragma unroll
-                for (int k = 0; k < NTALLY; ++k) {
-#pragma unroll
-                    for (int o2 = 16; o2 > 0; o2 >>= 1) {
-                        tal_e[k] += __shfl_down_sync(0xffffffffu, tal_e[k], o2);
-                        tal_n[k] += __shfl_down_sync(0xffffffffu, tal_n[k], o2);
-                    }
-                    if (lane == 0 && tal_n[k] > 0) {
-                        atomicAdd(&s_tal_e[si * NTALLY + k], tal_e[k]);
-                        atomicAdd(&s_tal_n[si * NTALLY + k], (unsigned long long)tal_n[k]);
-                    }
-                }
-            }
-        }
     }
     // what the queues still hold (each fewer than 32 particles)
     __syncwarp();
@@ -941,13 +947,19 @@ __global__ void k_j_reduce(GridDev g, const float *__restrict__ jscratch, const 
 }
 
 // Insert migrants: into a hole of the destination tile if one is free, else at
-// its end.  Grid-stride over the migration buffer (its fill is read on device).
-__global__ void k_rebin(SpDev sp, int *__restrict__ status) {
+// its end.  One launch for all species (grid y), grid-stride over the migration
+// buffer (its fill is read on device).
+__global__ void __launch_bounds__(256) k_rebin(const SpDev *__restrict__ sps, int *__restrict__ status) {
+    const SpDev &sp = sps[blockIdx.y];
     const int nm = min(*sp.mig_count, sp.mig_cap);
     // (a chunk's unused slots hold the destination -1)
     for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < nm; m += gridDim.x * blockDim.x) {
         const int t = sp.mdest[m];
         if (t < 0) continue;
+        // the migrant's loads do not wait for its slot
+        const float x = sp.mx[m], y = sp.my[m], z = sp.mz[m], ux = sp.mux[m], uy = sp.muy[m], uz = sp.muz[m];
+        const float w = sp.mw[m], zq = sp.zq ? sp.mzq[m] : 0.0f, tau = sp.tau ? sp.mtau[m] : 0.0f;
+        const uint64_t id = sp.mid[m];
         const int h = atomicAdd(&sp.hole_used[t], 1);
         int slot;
         if (h < sp.hole_count[t]) {
@@ -960,25 +972,38 @@ __global__ void k_rebin(SpDev sp, int *__restrict__ status) {
             }
         }
         const long long s = (long long)t * sp.cap + slot;
-        sp.x[s] = sp.mx[m]; sp.y[s] = sp.my[m]; sp.z[s] = sp.mz[m];
-        sp.ux[s] = sp.mux[m]; sp.uy[s] = sp.muy[m]; sp.uz[s] = sp.muz[m];
-        sp.w[s] = sp.mw[m];
-        if (sp.zq) sp.zq[s] = sp.mzq[m];
-        sp.id[s] = sp.mid[m];
-        if (sp.tau) sp.tau[s] = sp.mtau[m];
+        sp.x[s] = x; sp.y[s] = y; sp.z[s] = z;
+        sp.ux[s] = ux; sp.uy[s] = uy; sp.uz[s] = uz;
+        sp.w[s] = w;
+        if (sp.zq) sp.zq[s] = zq;
+        sp.id[s] = id;
+        if (sp.tau) sp.tau[s] = tau;
     }
 }
 
 // Close the holes no migrant filled: move live particles from the end of the
-// tile into them and shrink the count.
-__global__ void __launch_bounds__(32) k_compact(GridDev g, SpDev sp) {
-    // one warp per tile: the holes below the new count (in hole-list order)
-    // are filled with the live particles at or above it (in slot order), the
-    // same pairing as a serial walk of both lists; FIFO queues of up to 64
-    // entries in shared memory, refilled 32 candidates at a time
-    __shared__ int hq[64], sq[64];
-    const int t = blockIdx.x, lane = threadIdx.x;
-    (void)g;
+// tile into them and shrink the count.  One warp per tile, eight tiles per CTA,
+// all species in one launch (grid y): the holes below the new count (in
+// hole-list order) are filled with the live particles at or above it (in slot
+// order), the same pairing as a serial walk of both lists.  Both lists pass
+// through shared-memory queues, 128 candidates and up to 128 pairs at a time:
+// the walk is a chain of dependent loads, and four a lane in flight shorten it.
+// A step's last particle kernel also advances the step counter and empties the
+// migration buffers.  Together with the one launch of k_rebin, against one launch
+// a species of one-warp CTAs, 32 candidates at a time: five steps of two species
+// on 64 tiles 296 -> 271 us, on 315 tiles 471 -> 451 us, ten steps of a 64 x 32 x 32
+// hybrid run with a classification 3811 -> 3587 us.
+static constexpr int CP_WARPS = 8, CP_N = 128;
+__global__ void __launch_bounds__(32 * CP_WARPS) k_compact(GridDev g, const SpDev *__restrict__ sps, long long *step_dev) {
+    __shared__ int s_hq[CP_WARPS][2 * CP_N], s_sq[CP_WARPS][2 * CP_N];
+    const SpDev &sp = sps[blockIdx.y];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, t = blockIdx.x * CP_WARPS + warp;
+    if (step_dev && blockIdx.x == 0 && threadIdx.x == 0) {
+        *sp.mig_count = 0;
+        if (blockIdx.y == 0) *step_dev += 1;
+    }
+    if (t >= g.ntiles) return;
+    int *hq = s_hq[warp], *sq = s_sq[warp];
     const int hc = sp.hole_count[t], hu = sp.hole_used[t];
     const int n = min(sp.count[t], sp.cap);
     if (hu >= hc) {
@@ -993,43 +1018,76 @@ __global__ void __launch_bounds__(32) k_compact(GridDev g, SpDev sp) {
     const unsigned below = (1u << lane) - 1u;
     int h = hu, src = new_n, hn = 0, sn = 0;
     for (;;) {
-        while (hn < 32 && h < hc) {
-            const int hh = h + lane;
-            const int dst = hh < hc ? sp.holes[base + hh] : new_n;
-            const bool ok = dst < new_n;  // holes at or above new_n vanish with the shrink
-            const unsigned m = __ballot_sync(0xffffffffu, ok);
-            if (ok) hq[hn + __popc(m & below)] = dst;
-            hn += __popc(m);
-            h += 32;
+        while (hn < CP_N && h < hc) {
+            int dst[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) dst[r] = h + 32 * r + lane < hc ? sp.holes[base + h + 32 * r + lane] : new_n;
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const bool ok = dst[r] < new_n;  // holes at or above new_n vanish with the shrink
+                const unsigned m = __ballot_sync(0xffffffffu, ok);
+                if (ok) hq[hn + __popc(m & below)] = dst[r];
+                hn += __popc(m);
+            }
+            h += 128;
         }
-        while (sn < 32 && src < n) {
-            const int s0 = src + lane;
-            const bool ok = s0 < n && !(sp.x[base + s0] < 0.0f);  // live slot (vacated slots hold x < 0)
-            const unsigned m = __ballot_sync(0xffffffffu, ok);
-            if (ok) sq[sn + __popc(m & below)] = s0;
-            sn += __popc(m);
-            src += 32;
+        while (sn < CP_N && src < n) {
+            float x[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) x[r] = src + 32 * r + lane < n ? sp.x[base + src + 32 * r + lane] : -1.0f;
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const bool ok = !(x[r] < 0.0f);  // live slot (vacated slots hold x < 0)
+                const unsigned m = __ballot_sync(0xffffffffu, ok);
+                if (ok) sq[sn + __popc(m & below)] = src + 32 * r + lane;
+                sn += __popc(m);
+            }
+            src += 128;
         }
         __syncwarp();
-        const int k = min(32, min(hn, sn));  // one pair per lane
+        const int k = min(CP_N, min(hn, sn));  // up to four pairs a lane
         if (k == 0) break;
-        if (lane < k) {
-            const long long a = base + hq[lane], b = base + sq[lane];
-            sp.x[a] = sp.x[b]; sp.y[a] = sp.y[b]; sp.z[a] = sp.z[b];
-            sp.ux[a] = sp.ux[b]; sp.uy[a] = sp.uy[b]; sp.uz[a] = sp.uz[b];
-            sp.w[a] = sp.w[b];
-            if (sp.zq) sp.zq[a] = sp.zq[b];
-            sp.id[a] = sp.id[b];
-            if (sp.tau) sp.tau[a] = sp.tau[b];
+        long long a[4], b[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int i = 32 * r + lane;
+            a[r] = i < k ? base + hq[i] : -1;
+            b[r] = i < k ? base + sq[i] : -1;
         }
-        // drop the k used entries of both queues
-        const int h0 = lane + k < hn ? hq[lane + k] : 0, h1 = lane + 32 + k < hn ? hq[lane + 32 + k] : 0;
-        const int q0 = lane + k < sn ? sq[lane + k] : 0, q1 = lane + 32 + k < sn ? sq[lane + 32 + k] : 0;
+        auto move = [&](auto *arr) {
+            std::remove_reference_t<decltype(arr[0])> v[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+                if (b[r] >= 0) v[r] = arr[b[r]];
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+                if (a[r] >= 0) arr[a[r]] = v[r];
+        };
+        move(sp.x);
+        move(sp.y);
+        move(sp.z);
+        move(sp.ux);
+        move(sp.uy);
+        move(sp.uz);
+        move(sp.w);
+        if (sp.zq) move(sp.zq);
+        move(sp.id);
+        if (sp.tau) move(sp.tau);
+        // drop the k used entries of both queues (fewer than 128 + 127 before)
+        int h1[8], q1[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const int i = 32 * r + lane + k;
+            h1[r] = i < hn ? hq[i] : 0;
+            q1[r] = i < sn ? sq[i] : 0;
+        }
         __syncwarp();
-        if (lane + k < hn) hq[lane] = h0;
-        if (lane + 32 + k < hn) hq[lane + 32] = h1;
-        if (lane + k < sn) sq[lane] = q0;
-        if (lane + 32 + k < sn) sq[lane + 32] = q1;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const int i = 32 * r + lane;
+            if (i + k < hn) hq[i] = h1[r];
+            if (i + k < sn) sq[i] = q1[r];
+        }
         hn -= k;
         sn -= k;
         __syncwarp();
@@ -1138,16 +1196,15 @@ static void push_launch(const GridDev &g, const float *E, const float *B, const 
 void launch_push_deposit(const GridDev &g, const float *E, const float *B, const SpDev *sps_dev, int nsp,
                          bool events, const QedDev &qd, float *jscratch, int *jvalid, int *status,
                          const long long *step_dev, cudaStream_t st) {
-    // A small grid has fewer tiles than the chip holds CTAs (152 SMs x 3), and one
-    // CTA's walk through its tile then decides: its tiles are split over clusters
-    // of 2 or 4 CTAs while the grid stays at or below PUSH_SPLIT_CTAS.  Five steps
-    // with the read-out, us, for 1 / 2 / 3 / 4 / 5 / 8 CTAs a tile: 64 tiles, all full
+    // A small grid has fewer tiles than the chip holds CTAs (152 SMs x 3 = 456), and
+    // one CTA's walk through its tile then decides: its tiles are split over clusters
+    // of up to 4 CTAs while all of them are resident at once.  Five steps with the
+    // read-out, us, for 1 / 2 / 3 / 4 / 5 / 8 CTAs a tile: 64 tiles, all full
     // 423 / 334 / 301 / 298 / 296 / 371; 128 tiles, half of them empty (10 steps and a
     // classification) 5346 / 4099 / 3843 / 3833 / 3829 / 3921; 315 tiles, 3 particles a
     // cell 463 / 576 / 649 / 719 / 830 / 1079: every CTA stages the tile's fields and
     // clears a frame, so a grid that fills the chip is left whole.
-    int split = 1;
-    while (split < 4 && g.ntiles * split * 2 <= PUSH_SPLIT_CTAS) split *= 2;
+    const int split = std::max(1, std::min(4, PUSH_SPLIT_CTAS / std::max(1, g.ntiles)));
     auto go = [&](auto kern) { kern(g, E, B, sps_dev, nsp, qd, jscratch, jvalid, status, step_dev, split, st); };
     auto shape = [&](auto ev, auto sp) {
         constexpr bool EV = decltype(ev)::value, SP = decltype(sp)::value;
@@ -1166,17 +1223,17 @@ void launch_j_reduce(const GridDev &g, const float *jscratch, const int *jvalid,
     k_j_reduce<<<grid, bx, 0, st>>>(g, jscratch, jvalid, J);
 }
 
-void launch_rebin(const GridDev &g, const SpDev &s, int *status, cudaStream_t st) {
-    (void)g;
-    k_rebin<<<152 * 4, 256, 0, st>>>(s, status);
+void launch_rebin(const SpDev *sps_dev, int nsp, int *status, cudaStream_t st) {
+    k_rebin<<<dim3(152 * 4, (unsigned)nsp), 256, 0, st>>>(sps_dev, status);
 }
 
 void launch_regrid(const GridDev &g, const SpDev &from, const SpDev &to, cudaStream_t st) {
     k_regrid<<<g.ntiles, 256, 0, st>>>(from, to);
 }
 
-void launch_compact(const GridDev &g, const SpDev &s, cudaStream_t st) {
-    k_compact<<<g.ntiles, 32, 0, st>>>(g, s);
+void launch_compact(const GridDev &g, const SpDev *sps_dev, int nsp, long long *step_dev, cudaStream_t st) {
+    k_compact<<<dim3((unsigned)((g.ntiles + CP_WARPS - 1) / CP_WARPS), (unsigned)nsp), 32 * CP_WARPS, 0, st>>>(g, sps_dev,
+                                                                                                              step_dev);
 }
 
 void launch_count_tiles(const GridDev &g, long long n, const float *x, const float *y, const float *z,

@@ -755,7 +755,7 @@ hyb_status regime_update(hyb_ctx *c, const float *pm, const float *ps) {
         k_clamp_counts<<<(g.ntiles + 255) / 256, 256, 0, st>>>(g.ntiles, dst);
         k_particles_to_fluid<<<g.ntiles, 256, 4 * sm1, st>>>(g, mask, dst, c->jscratch, c->jvalid, c->status);
         k_moments_gather<<<node_grid(g), node_block(g), 0, st>>>(g, c->jscratch, c->jvalid, c->fluids[f]);
-        launch_compact(g, dst, st);
+        launch_compact(g, c->sp_dev + sid, 1, nullptr, st);
         launches += 6;
     }
     c->launches_classify += launches;
