@@ -82,6 +82,32 @@ def test_tiles_that_empty_and_fill(arena, n):
     sim.close()
 
 
+# rows shorter than a block of 32 nodes, and ending inside one; one fluid, and two (the second one's loads run ahead)
+@pytest.mark.parametrize("size", [(4, 4, 4), (36, 8, 4)])
+@pytest.mark.parametrize("nf", [1, 2])
+def test_fluid_blocks_match_oracle(size, nf):
+    nx, ny, nz = size
+    rng = np.random.default_rng(nf)
+    inp = dict(grid=dict(nx=nx, ny=ny, nz=nz, dx=0.35), species=[],
+               E=(0.02 * rng.standard_normal((3, nz, ny, nx))).astype(np.float32),
+               B=(0.02 * rng.standard_normal((3, nz, ny, nx))).astype(np.float32))
+    sim, orc = make_pair(inp, tile=4)
+    for q in range(nf):
+        fl = dict(q=-1.0 if q == 0 else 1.0, m=1.0 if q == 0 else 100.0,
+                  n=rng.uniform(0.4, 0.6, (nz, ny, nx)).astype(np.float32),
+                  **{c: (0.05 * rng.standard_normal((nz, ny, nx))).astype(np.float32) for c in ("ux", "uy", "uz")})
+        sim.load_fluid(**fl)
+        orc.load_fluid(**fl)
+    sim.step(4)
+    orc.step(4)
+    for q in range(nf):
+        g, o = sim.get_fluid(q), orc.fluids[q]
+        # four steps of some fifty FP32 operations a node, 6e-8 each
+        assert rel_l2(g["n"], o.n) <= 1e-5
+        assert rel_l2(np.stack([g["ux"], g["uy"], g["uz"]]), o.u) <= 1e-4
+    sim.close()
+
+
 # W = 8 and 16: one tile; 24, 40: several, the last one ragged; one plane, and more planes than a column's start
 @pytest.mark.parametrize("shape", [(3, 1, 32, 40), (2, 5, 16, 16), (1, 33, 16, 48)])
 def test_classifier_ragged_volumes_match_oracle(shape):
