@@ -237,23 +237,22 @@ __device__ __forceinline__ void deposit_one_crossing(unsigned *__restrict__ sj, 
     const int Jc = base + c * G3, Jp = base + sel3(c, 1, 2, 0) * G3, Jq = base + sel3(c, 2, 0, 1) * G3;
     const float fc = A.w * sel3(c, jfac[0], jfac[1], jfac[2]), fp = A.w * sel3(c, jfac[1], jfac[2], jfac[0]),
                 fq = A.w * sel3(c, jfac[2], jfac[0], jfac[1]);
-    {
-        int idx[8];
-        float val[8];
 #pragma unroll
-        for (int bq = 0; bq < 2; ++bq)
+    for (int bq = 0; bq < 2; ++bq) {
+        int idx[4];
+        float val[4];
 #pragma unroll
-            for (int bp = 0; bp < 2; ++bp) {
-                const float w = esirkepov_cross(s0p[bp], dp[bp], s0q[bq], dq[bq]);
-                float acc = 0.0f;
+        for (int bp = 0; bp < 2; ++bp) {
+            const float w = esirkepov_cross(s0p[bp], dp[bp], s0q[bq], dq[bq]);
+            float acc = 0.0f;
 #pragma unroll
-                for (int a = 0; a < 2; ++a) {
-                    acc += dc[a] * w;
-                    idx[(bq * 2 + bp) * 2 + a] = Jc + a * sc + bp * sp + bq * sq;
-                    val[(bq * 2 + bp) * 2 + a] = fc * acc;
-                }
+            for (int a = 0; a < 2; ++a) {
+                acc += dc[a] * w;
+                idx[bp * 2 + a] = Jc + a * sc + bp * sp + bq * sq;
+                val[bp * 2 + a] = fc * acc;
             }
-        fix_add<8, false>(sj, 3 * G3, idx, val);
+        }
+        fix_add<4, false>(sj, 3 * G3, idx, val);
     }
     {
         // along p: transverse axes q (two nodes) and c (three)
@@ -409,7 +408,14 @@ __device__ __forceinline__ void deposit_quadratic(unsigned *__restrict__ sj, con
 
 // A warp's queue of crossing particles, 32 entries in shared memory: `n` of
 // them are taken (warp-uniform).  The lanes in `want` append; a full queue is
-// handed to `flush` with every lane of the warp holding one entry.
+// handed to `flush` with every lane of the warp holding one entry.  The entries
+// that did not fit go in before `flush` runs, so that their eight values are dead
+// in its long code: held across it (and with eight sums of the one-axis stencil
+// in flight instead of four) they made the compiler spill the next particle's
+// prefetched values, and a spill waits for the load it stores -- every particle
+// pass then paid the memory latency the prefetch is there to hide.  One launch,
+// 15.7 M particles at rest 623 -> 439 us, slow (|u| ~ 1e-3, hardly any crossing)
+// 678 -> 501 us, thermal 881 -> 727 us.
 template <class F>
 __device__ __forceinline__ void queue_put(float4 *qa, int &n, bool want, const float4 A, const float4 B, int lane,
                                           F flush) {
@@ -424,13 +430,14 @@ __device__ __forceinline__ void queue_put(float4 *qa, int &n, bool want, const f
     n += __popc(m);
     if (n >= PUSH_Q) {
         __syncwarp();
-        flush(qa[lane], qb[lane]);
+        const float4 ea = qa[lane], eb = qb[lane];
         __syncwarp();
         n -= PUSH_Q;
         if (want && pos >= PUSH_Q) {
             qa[pos - PUSH_Q] = A;
             qb[pos - PUSH_Q] = B;
         }
+        flush(ea, eb);
     }
 }
 
