@@ -636,13 +636,13 @@ hyb_status hyb_surrogate_forward(hyb_surrogate *m, const float *x, int B, int D,
 hyb_status hyb_surrogate_mc(hyb_surrogate *m, const float *x, int B, int D, int H, int W, float *pm, float *ps) {
     if (!m || !x || !pm || !ps) return set_error(HYB_EINVAL, "null argument");
     hyb_status s = check_shape(B, D, H, W);
+    if (s != HYB_OK) return s;  // (an empty volume among them: the division below needs cells)
     const long long V = (long long)D * H * W, cells = (long long)B * V;
     // as many passes side by side as keep a launch's volume within MC_CELLS: a small
     // batch does not fill the SMs (65 536 cells: four passes, 6.3 -> 1.9 ms for 16)
     const int K = m->d.mc_passes;
     const int G = (int)std::max<long long>(1, std::min<long long>(K, MC_CELLS / cells));
-    if (s == HYB_OK) s = reserve(m, cells * G);
-    if (s != HYB_OK) return s;
+    if ((s = reserve(m, cells * G)) != HYB_OK) return s;
     k_sur_prep<<<nbk(cells), RB, 0, m->stream>>>(x, B, V, m->mean, m->std_, m->a[0]);
     if ((s = forward(m, 0, DROP_LAYER - 1, B, D, H, W, -1, 1, false)) != HYB_OK) return s;
     for (int k = 0; k < K; k += G) {
