@@ -423,7 +423,9 @@ hyb_status hyb_surrogate_forward(hyb_surrogate *s, const float *x_dev, int batch
                                  float *y_dev);
 /* Monte Carlo dropout: mc_passes passes (pass index 0 .. mc_passes - 1);
  * mean and population standard deviation of the de-normalised prediction
- * per value (device FP32, layout of x).  Stream-ordered. */
+ * per value (device FP32, layout of x).  Stream-ordered.  Passes of a small
+ * batch run side by side, up to 262 144 cells together (1.2 KB a cell), or
+ * fewer where the device memory does not hold them. */
 hyb_status hyb_surrogate_mc(hyb_surrogate *s, const float *x_dev, int batch, int D, int H, int W, float *mean_dev,
                             float *std_dev);
 typedef struct {

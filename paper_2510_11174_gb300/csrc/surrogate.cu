@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "conv_tc.cuh"
+#include "mc_passes.h"
 #include "hyb_internal.cuh"
 #include "philox.cuh"
 
@@ -316,9 +317,12 @@ struct hyb_surrogate {
     __nv_bfloat16 *pk[SL] = {}, *pkT[SL] = {};        // channel-chunk packs (forward, data gradient)
     float *mean = nullptr, *std_ = nullptr, *dstd = nullptr;  // dstd: unit of the predicted change
     int *status = nullptr;
-    long long cap = 0;                                // cells the activation buffers hold
+    // cells the buffers hold: the inputs of the layers that the MC passes share (a[0], a[1]),
+    // what every pass of a forward has of its own (the other a, y, the s of layers in several
+    // chunks), and what only a training step needs (the other s, G, dz)
+    long long cap_in = 0, cap_pass = 0, cap_train = 0;
     __nv_bfloat16 *a[SL] = {};                        // a[l]: input of layer l, [cells][CIP[l]]
-    float *s[SL] = {};                                // pre-activation sums of layer l (no bias), [cells][COP[l]]
+    float *s[SL - 1] = {};                            // pre-activation sums of layer l (no bias), [cells][COP[l]]
     float *G[SL + 1] = {};                            // G[l]: dL/d a[l] ([cells][CIP[l]]), G[SL] = dL/dy
     float *y = nullptr;                               // prediction [cells][16] (normalised)
     __nv_bfloat16 *dz = nullptr;                      // data gradient of the current layer, [cells][<= 128]
@@ -360,32 +364,50 @@ hyb_status repack(hyb_surrogate *m) {
     return HYB_OK;
 }
 
-hyb_status reserve(hyb_surrogate *m, long long cells) {
-    if (cells <= m->cap) return HYB_OK;
+struct Buf {
+    void **p;
+    size_t cell;  // bytes per cell
+};
+
+// Buffers of `cap` cells replaced by larger ones.  If one does not fit, none is
+// kept (cap = 0) and the CUDA error is cleared: the caller may ask for fewer.
+hyb_status grow(hyb_surrogate *m, long long &cap, long long cells, const std::vector<Buf> &bufs) {
+    if (cells <= cap) return HYB_OK;
     cudaStreamSynchronize(m->stream);  // buffers are replaced only between stream-ordered uses
-    for (int l = 0; l < SL; ++l) {
-        s_free(m, m->a[l]);
-        s_free(m, m->s[l]);
-        m->a[l] = nullptr;
-        m->s[l] = nullptr;
-    }
-    for (int l = 0; l <= SL; ++l) {
-        s_free(m, m->G[l]);
-        m->G[l] = nullptr;
-    }
-    s_free(m, m->y);
-    s_free(m, m->dz);
-    m->cap = 0;
-    for (int l = 0; l < SL; ++l)
-        if (s_alloc(m, (void **)&m->a[l], sizeof(__nv_bfloat16) * CIP[l] * cells) ||
-            s_alloc(m, (void **)&m->s[l], sizeof(float) * COP[l] * cells) ||
-            (l > 0 && s_alloc(m, (void **)&m->G[l], sizeof(float) * CIP[l] * cells)))
+    auto drop = [&]() {
+        for (const Buf &b : bufs) {
+            s_free(m, *b.p);
+            *b.p = nullptr;
+        }
+        cap = 0;
+    };
+    drop();
+    for (const Buf &b : bufs)
+        if (s_alloc(m, b.p, b.cell * (size_t)cells)) {
+            *b.p = nullptr;
+            drop();
+            cudaGetLastError();
             return set_error(HYB_ENOMEM, "surrogate activation buffers");
-    if (s_alloc(m, (void **)&m->G[SL], sizeof(float) * 16 * cells) || s_alloc(m, (void **)&m->y, sizeof(float) * 16 * cells) ||
-        s_alloc(m, (void **)&m->dz, sizeof(__nv_bfloat16) * 128 * cells))
-        return set_error(HYB_ENOMEM, "surrogate activation buffers");
-    m->cap = cells;
+        }
+    cap = cells;
     return HYB_OK;
+}
+
+// buffers for `passes` forward passes of a batch of `cells` cells side by side (1.2 KB a
+// cell and pass), and for a training step of it (2 KB a cell)
+hyb_status reserve(hyb_surrogate *m, long long cells, int passes, bool train) {
+    std::vector<Buf> in, pass, tr;
+    for (int l = 0; l < SL; ++l)
+        (l <= DROP_LAYER ? in : pass).push_back({(void **)&m->a[l], sizeof(__nv_bfloat16) * CIP[l]});
+    for (int l = 0; l < SL - 1; ++l)
+        (CIP[l] > chunk_of(CIP[l]) ? pass : tr).push_back({(void **)&m->s[l], sizeof(float) * COP[l]});
+    pass.push_back({(void **)&m->y, sizeof(float) * 16});
+    for (int l = 1; l <= SL; ++l) tr.push_back({(void **)&m->G[l], sizeof(float) * (l < SL ? CIP[l] : 16)});
+    tr.push_back({(void **)&m->dz, sizeof(__nv_bfloat16) * 128});
+    hyb_status s = grow(m, m->cap_in, cells, in);
+    if (s == HYB_OK) s = grow(m, m->cap_pass, cells * passes, pass);
+    if (s == HYB_OK && train) s = grow(m, m->cap_train, cells, tr);
+    return s;
 }
 
 // conv(x [cells][nin]; the packs pk) -> nout channels: one launch per input-channel
@@ -464,8 +486,8 @@ hyb_status forward(hyb_surrogate *m, int first, int last, int B, int D, int H, i
                 a.pass_b = B;
             }
         }
-        const hyb_status st = conv_chunks(m, m->a[l], CIP[l], m->pk[l], COP[l], m->s[l], train && l < SL - 1, a,
-                                          shared ? B : B * groups, D, H, W);
+        const hyb_status st = conv_chunks(m, m->a[l], CIP[l], m->pk[l], COP[l], l < SL - 1 ? m->s[l] : nullptr,
+                                          train && l < SL - 1, a, shared ? B : B * groups, D, H, W);
         if (st != HYB_OK) return st;
     }
     return HYB_OK;
@@ -624,7 +646,7 @@ hyb_status hyb_surrogate_forward(hyb_surrogate *m, const float *x, int B, int D,
     if (!m || !x || !y) return set_error(HYB_EINVAL, "null argument");
     hyb_status s = check_shape(B, D, H, W);
     const long long V = (long long)D * H * W, cells = (long long)B * V;
-    if (s == HYB_OK) s = reserve(m, cells);
+    if (s == HYB_OK) s = reserve(m, cells, 1, false);
     if (s != HYB_OK) return s;
     k_sur_prep<<<nbk(cells), RB, 0, m->stream>>>(x, B, V, m->mean, m->std_, m->a[0]);
     if ((s = forward(m, 0, SL - 1, B, D, H, W, pass, 1, false)) != HYB_OK) return s;
@@ -638,11 +660,9 @@ hyb_status hyb_surrogate_mc(hyb_surrogate *m, const float *x, int B, int D, int 
     hyb_status s = check_shape(B, D, H, W);
     if (s != HYB_OK) return s;  // (an empty volume among them: the division below needs cells)
     const long long V = (long long)D * H * W, cells = (long long)B * V;
-    // as many passes side by side as keep a launch's volume within MC_CELLS: a small
-    // batch does not fill the SMs (65 536 cells: four passes, 6.3 -> 1.9 ms for 16)
     const int K = m->d.mc_passes;
-    const int G = (int)std::max<long long>(1, std::min<long long>(K, MC_CELLS / cells));
-    if ((s = reserve(m, cells * G)) != HYB_OK) return s;
+    const int G = passes_side_by_side(K, cells, MC_CELLS, [&](int g) { return s = reserve(m, cells, g, false); });
+    if (s != HYB_OK) return s;
     k_sur_prep<<<nbk(cells), RB, 0, m->stream>>>(x, B, V, m->mean, m->std_, m->a[0]);
     if ((s = forward(m, 0, DROP_LAYER - 1, B, D, H, W, -1, 1, false)) != HYB_OK) return s;
     for (int k = 0; k < K; k += G) {
@@ -660,7 +680,7 @@ hyb_status hyb_surrogate_train_step(hyb_surrogate *m, const float *x, const floa
     if (!m || !x || !tg || !out) return set_error(HYB_EINVAL, "null argument");
     hyb_status s = check_shape(B, D, H, W);
     const long long V = (long long)D * H * W, cells = (long long)B * V;
-    if (s == HYB_OK) s = reserve(m, cells);
+    if (s == HYB_OK) s = reserve(m, cells, 1, true);
     if (s != HYB_OK) return s;
     if (B > m->ecap) {
         s_free(m, m->epart);
