@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "hyb_internal.cuh"
+#include "push_shape.h"
 
 namespace hyb {
 
@@ -84,7 +85,7 @@ static void enqueue_step(hyb_ctx *c) {
         for (int i = 0; i < set.n; ++i)
             events = events || set.s[i].zmax > 0 || set.s[i].qed || (set.s[i].kind == HYB_KIND_PHOTON && set.s[i].pair_e >= 0);
         launch_push_deposit(g, c->E, c->B, c->sp_dev, set.n, events, c->qed, c->jscratch, c->jvalid, c->status, c->step_dev,
-                            st);
+                            push_split(g.T, g.order, g.ntiles, c->sms), st);
         pm.end(HYB_PH_PUSH);
         pm.begin(HYB_PH_JREDUCE);
         launch_j_reduce(g, c->jscratch, c->jvalid, c->J, st);
@@ -250,6 +251,10 @@ hyb_status hyb_init_grid(const hyb_grid_desc *d, hyb_ctx **out) {
         }
         c->own_stream = true;
     }
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0)
+        c->sms = sms;
     if (d->arena_dev) {
         c->arena.base = (char *)d->arena_dev;
         c->arena.size = d->arena_bytes;

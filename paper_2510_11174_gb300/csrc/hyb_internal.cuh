@@ -243,6 +243,7 @@ struct Arena {
 struct hyb_ctx {
     hyb_grid_desc desc;
     hyb::GridDev g;
+    int sms = 152;               // SMs of the device
     cudaStream_t stream;
     bool own_stream = false;
     bool error_latched = false;  // set when a synchronising call saw a device error
@@ -340,10 +341,10 @@ void launch_laser_source(const GridDev &g, const hyb_grid_desc &d, const float *
 void launch_step_inc(long long *step_dev, cudaStream_t st);
 void launch_wait_selftest(long long polls, int *status, cudaStream_t st);
 
-// events: some species ionizes, emits photons or creates pairs
+// events: some species ionizes, emits photons or creates pairs; split: CTAs per tile (push_shape.h)
 void launch_push_deposit(const GridDev &g, const float *E, const float *B, const SpDev *sps_dev, int nsp,
                          bool events, const QedDev &qd, float *jscratch, int *jvalid, int *status, const long long *step_dev,
-                         cudaStream_t st);
+                         int split, cudaStream_t st);
 hyb_status setup_qed(hyb_ctx *c);  // builds the QED tables once per context
 hyb_status regime_update(hyb_ctx *c, const float *p_mean, const float *p_std);
 // the x-range [*xa, *xb) of nodes within `reach` nodes (along x) of an

@@ -30,6 +30,7 @@
 #include "philox.cuh"
 #include "qed.cuh"
 #include "particles.cuh"
+#include "push_shape.h"
 
 #include <cooperative_groups.h>
 
@@ -43,23 +44,23 @@ namespace cg = cooperative_groups;
 // field frame edge: a shape of order k gathers from k nodes below the tile to k - 1 above it
 __host__ __device__ constexpr int frame_F(int T, int order = 1) { return T + 2 * order; }
 
-// 8^3 tiles hold thousands of particles, 4^3 tiles a few hundred: smaller CTAs
-// there leave fewer lanes idle in a species' last pass and fewer warps waiting
-__host__ __device__ constexpr int push_threads(int T) { return T == 8 ? 256 : 128; }
-// CTAs per SM by shared memory (8^3: 73 KB linear, 114 KB quadratic shape; 4^3: 25 and 42 KB) and registers
-__host__ __device__ constexpr int push_ctas(int T, int order) { return T == 8 ? (order == 1 ? 3 : 2) : (order == 1 ? 6 : 5); }
 static constexpr int PUSH_Q = 32;          // entries of a per-warp queue of cell-crossing particles
-static constexpr int PUSH_SPLIT_CTAS = 456;   // see launch_push_deposit
 
 __host__ __device__ constexpr size_t align16(size_t b) { return (b + 15) & ~(size_t)15; }
 
 // the current frame (3 components, 64-bit fixed point), the fields, the
 // per-warp queues (two of PUSH_Q entries of two float4), the species
-size_t push_smem_bytes(int T, int order, int nsp) {
+constexpr size_t push_smem_bytes(int T, int order, int nsp) {
     const int F = frame_F(T, order), G = frame_G(T, order);
     return align16(sizeof(unsigned long long) * 3 * (size_t)G * G * G) + align16(sizeof(float) * 6 * (size_t)F * F * F) +
            sizeof(float4) * (push_threads(T) / 32) * 4 * PUSH_Q + sizeof(SpDev) * (size_t)nsp;
 }
+// push_ctas() of them fit an SM's 228 KB with every species loaded (1 KB a CTA is
+// the system's, 1 KB holds the kernel's static arrays)
+constexpr bool push_fits(int T, int order) {
+    return (push_smem_bytes(T, order, HYB_MAX_SPECIES) + 2048) * push_ctas(T, order) <= 228 * 1024;
+}
+static_assert(push_fits(8, 1) && push_fits(8, 2) && push_fits(4, 1) && push_fits(4, 2), "push_ctas");
 
 // CIC base index and weight of one axis on the integer (i) and the
 // half-integer (h) grid, relative to the frame origin o (global node index of
@@ -1202,16 +1203,7 @@ static void push_launch(const GridDev &g, const float *E, const float *B, const 
 
 void launch_push_deposit(const GridDev &g, const float *E, const float *B, const SpDev *sps_dev, int nsp,
                          bool events, const QedDev &qd, float *jscratch, int *jvalid, int *status,
-                         const long long *step_dev, cudaStream_t st) {
-    // A small grid has fewer tiles than the chip holds CTAs (152 SMs x 3 = 456), and
-    // one CTA's walk through its tile then decides: its tiles are split over clusters
-    // of up to 4 CTAs while all of them are resident at once.  Five steps with the
-    // read-out, us, for 1 / 2 / 3 / 4 / 5 / 8 CTAs a tile: 64 tiles, all full
-    // 423 / 334 / 301 / 298 / 296 / 371; 128 tiles, half of them empty (10 steps and a
-    // classification) 5346 / 4099 / 3843 / 3833 / 3829 / 3921; 315 tiles, 3 particles a
-    // cell 463 / 576 / 649 / 719 / 830 / 1079: every CTA stages the tile's fields and
-    // clears a frame, so a grid that fills the chip is left whole.
-    const int split = std::max(1, std::min(4, PUSH_SPLIT_CTAS / std::max(1, g.ntiles)));
+                         const long long *step_dev, int split, cudaStream_t st) {
     auto go = [&](auto kern) { kern(g, E, B, sps_dev, nsp, qd, jscratch, jvalid, status, step_dev, split, st); };
     auto shape = [&](auto ev, auto sp) {
         constexpr bool EV = decltype(ev)::value, SP = decltype(sp)::value;
