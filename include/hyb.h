@@ -526,7 +526,10 @@ hyb_status hyb_step(hyb_ctx *ctx, int nsteps);
  * a context before and after stay ordered.  Capacity growth works as in
  * hyb_step.  Contexts must be distinct and on the current device; a context
  * may belong to several batches but must not be stepped by two at once.  The
- * batch does not own its contexts: destroy it before them. */
+ * batch does not own its contexts: destroy it before them.  The SMs are shared
+ * by the tiles of all contexts: from then on each context's push takes the CTAs
+ * a tile that suit the largest batch it was put in (the results do not depend
+ * on it). */
 typedef struct hyb_batch hyb_batch;
 hyb_status hyb_batch_create(hyb_ctx *const *ctxs, int n, void *stream, hyb_batch **out);
 hyb_status hyb_batch_step(hyb_batch *batch, int nsteps);

@@ -72,6 +72,11 @@ struct PhaseMark {
     }
 };
 
+// CTAs per tile of the context's push
+static int ctx_split(const hyb_ctx *c) {
+    return push_split(c->g.T, c->g.order, std::max<long long>(c->g.ntiles, c->batch_tiles), c->sms);
+}
+
 // Enqueue one full step on the context stream.
 static void enqueue_step(hyb_ctx *c) {
     const GridDev &g = c->g;
@@ -85,7 +90,7 @@ static void enqueue_step(hyb_ctx *c) {
         for (int i = 0; i < set.n; ++i)
             events = events || set.s[i].zmax > 0 || set.s[i].qed || (set.s[i].kind == HYB_KIND_PHOTON && set.s[i].pair_e >= 0);
         launch_push_deposit(g, c->E, c->B, c->sp_dev, set.n, events, c->qed, c->jscratch, c->jvalid, c->status, c->step_dev,
-                            push_split(g.T, g.order, g.ntiles, c->sms), st);
+                            ctx_split(c), st);
         pm.end(HYB_PH_PUSH);
         pm.begin(HYB_PH_JREDUCE);
         launch_j_reduce(g, c->jscratch, c->jvalid, c->J, st);
@@ -911,6 +916,14 @@ hyb_status hyb_batch_create(hyb_ctx *const *ctxs, int n, void *stream, hyb_batch
     if (!ok) {
         hyb_batch_destroy(b);
         return set_error(HYB_ECUDA, "batch stream or events");
+    }
+    // the branches push at the same time: each context's share of the SMs decides how far its tiles are split
+    long long tiles = 0;
+    for (hyb_ctx *c : b->ctx) tiles += c->g.ntiles;
+    for (hyb_ctx *c : b->ctx) {
+        const int before = ctx_split(c);
+        c->batch_tiles = std::max(c->batch_tiles, tiles);
+        if (ctx_split(c) != before) c->graph_valid = false;
     }
     *out = b;
     return HYB_OK;

@@ -244,6 +244,7 @@ struct hyb_ctx {
     hyb_grid_desc desc;
     hyb::GridDev g;
     int sms = 152;               // SMs of the device
+    long long batch_tiles = 0;   // tiles of the largest batch the context is in (they step at the same time)
     cudaStream_t stream;
     bool own_stream = false;
     bool error_latched = false;  // set when a synchronising call saw a device error

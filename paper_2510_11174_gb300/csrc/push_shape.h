@@ -14,6 +14,7 @@ constexpr int push_ctas(int T, int order) { return T == 8 ? (order == 1 ? 3 : 2)
 // push_ctas), and one CTA's walk through its tile then decides: its tiles are split
 // over clusters of up to 4 CTAs while all of them are resident at once.  Every CTA
 // stages the tile's fields and clears a frame, so what fills the chip is left whole.
+// `tiles` counts the tiles of every context that steps at the same time (a batch).
 // One step, us, for 1 / 2 / 3 / 4 CTAs a tile on 152 SMs (* this rule's choice):
 //   8^3 linear (456 resident)     80 tiles 153 / 122 / 104 / 104*   144 tiles 137 / 117 / 114* / 139
 //                                216 tiles 167 / 141* / 173 / 164
@@ -23,6 +24,8 @@ constexpr int push_ctas(int T, int order) { return T == 8 ? (order == 1 ? 3 : 2)
 //                                343 tiles 74 / 70* / 84 / 84       512 tiles 83* / 94 / 99 / 108
 //   4^3 quadratic (760)          216 tiles 114 / 105 / 99* / 112    343 tiles 141 / 137* / 143 / 134
 //                                512 tiles 177* / 200 / 203 / 193
+//   batches of 64-tile 8^3 runs  2 runs 144 / 124 / 124* / 136      4 runs 192* / 208 / 204 / 209
+//                                8 runs 335* / 347 / 362 / 367      16 runs 896* / 951 / 1019 / 1023
 constexpr int push_split(int T, int order, long long tiles, int sms) {
     const long long fit = tiles > 0 ? (long long)sms * push_ctas(T, order) / tiles : 1;
     return fit < 1 ? 1 : (fit > 4 ? 4 : (int)fit);

@@ -45,3 +45,8 @@ def test_tiles_are_split_while_all_ctas_are_resident(rule, T, order, sms):
 def test_quadratic_8_tiles_count_two_ctas_an_sm(rule):
     """153 to 228 tiles of the quadratic shape fill the 304 resident CTAs: they are not split."""
     assert [s for s, _ in rule([(8, 2, n, 152) for n in (76, 77, 152, 153, 228)])] == [4, 3, 2, 1, 1]
+
+
+def test_batches_count_the_tiles_of_all_their_contexts(rule):
+    """1, 2, 4 and 8 contexts of 64 tiles side by side: 4, 3, 1 and 1 CTAs a tile."""
+    assert [s for s, _ in rule([(8, 1, 64 * n, 152) for n in (1, 2, 4, 8)])] == [4, 3, 1, 1]
