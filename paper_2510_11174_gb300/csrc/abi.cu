@@ -132,6 +132,35 @@ static void enqueue_step(hyb_ctx *c) {
     c->launches_per_step = k;
 }
 
+static void ctx_free(hyb_ctx *c, void *p);
+
+// the migration buffer of a species: `mig` slots and, with chunks, room for the
+// slots the push's warps leave unused in their last chunks
+static hyb_status alloc_migration(hyb_ctx *c, SpDev &s, long long mig, bool chunks, bool has_zq, bool has_tau) {
+    const GridDev &g = c->g;
+    s.mig_chunks = chunks ? 1 : 0;
+    if (chunks) mig += MIG_CHUNK * push_warps(g.T, g.order, g.ntiles, c->sms);
+    s.mig_cap = (int)std::min<long long>(mig, 0x7fffffffLL);
+    const struct {
+        void **p;
+        size_t bytes;
+    } bufs[] = {{(void **)&s.mx, sizeof(float)},   {(void **)&s.my, sizeof(float)},   {(void **)&s.mz, sizeof(float)},
+                {(void **)&s.mux, sizeof(float)},  {(void **)&s.muy, sizeof(float)},  {(void **)&s.muz, sizeof(float)},
+                {(void **)&s.mw, sizeof(float)},   {(void **)&s.mid, sizeof(uint64_t)}, {(void **)&s.mdest, sizeof(int)},
+                {(void **)&s.mzq, has_zq ? sizeof(float) : 0}, {(void **)&s.mtau, has_tau ? sizeof(float) : 0}};
+    for (const auto &b : bufs) *b.p = nullptr;
+    for (const auto &b : bufs)
+        if (b.bytes && ctx_alloc(c, b.p, b.bytes * s.mig_cap)) {
+            *b.p = nullptr;
+            for (const auto &f : bufs) {
+                ctx_free(c, *f.p);
+                *f.p = nullptr;
+            }
+            return HYB_ENOMEM;
+        }
+    return HYB_OK;
+}
+
 // the per-slot arrays (particles, hole list) and the migration buffer of a
 // species with `cap` slots per tile
 hyb_status alloc_slots(hyb_ctx *c, SpDev &s, int cap, bool has_zq, bool has_tau) {
@@ -146,22 +175,12 @@ hyb_status alloc_slots(hyb_ctx *c, SpDev &s, int cap, bool has_zq, bool has_tau)
     if (ctx_alloc(c, (void **)&s.id, sizeof(uint64_t) * slots) || ctx_alloc(c, (void **)&s.holes, sizeof(int) * slots))
         return HYB_ENOMEM;
     // a particle moves less than one cell per step, so only the shell of a tile can leave it
-    long long mig = std::min<long long>((long long)slots, std::max<long long>(65536, (long long)slots / 2));
-    // room for the slots the push's warps leave unused in their last chunks: 8 warps a tile, of up to 4 CTAs a
-    // tile on grids small enough to be split.  A caller's arena was sized without it: no chunks there.
-    s.mig_chunks = c->arena.base ? 0 : 1;
-    if (s.mig_chunks)
-        mig += MIG_CHUNK * 8LL * std::max<long long>(c->g.ntiles, std::min<long long>(4LL * c->g.ntiles, 512));
-    s.mig_cap = (int)std::min<long long>(mig, 0x7fffffffLL);
-    float **ml[7] = {&s.mx, &s.my, &s.mz, &s.mux, &s.muy, &s.muz, &s.mw};
-    for (auto f : ml)
-        if (ctx_alloc(c, (void **)f, sizeof(float) * s.mig_cap)) return HYB_ENOMEM;
-    if (has_zq && ctx_alloc(c, (void **)&s.mzq, sizeof(float) * s.mig_cap)) return HYB_ENOMEM;
-    if (has_tau && ctx_alloc(c, (void **)&s.mtau, sizeof(float) * s.mig_cap)) return HYB_ENOMEM;
-    if (ctx_alloc(c, (void **)&s.mid, sizeof(uint64_t) * s.mig_cap) ||
-        ctx_alloc(c, (void **)&s.mdest, sizeof(int) * s.mig_cap))
-        return HYB_ENOMEM;
-    return HYB_OK;
+    const long long mig = std::min<long long>((long long)slots, std::max<long long>(65536, (long long)slots / 2));
+    // A caller's arena was sized without room for chunks: none there, nor where the device has no memory for it.
+    if (c->arena.base) return alloc_migration(c, s, mig, false, has_zq, has_tau);
+    if (alloc_migration(c, s, mig, true, has_zq, has_tau) == HYB_OK) return HYB_OK;
+    cudaGetLastError();
+    return alloc_migration(c, s, mig, false, has_zq, has_tau);
 }
 
 // release a buffer of the context (buffers carved from a caller's arena stay

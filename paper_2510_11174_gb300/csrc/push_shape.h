@@ -31,4 +31,9 @@ constexpr int push_split(int T, int order, long long tiles, int sms) {
     return fit < 1 ? 1 : (fit > 4 ? 4 : (int)fit);
 }
 
+// warps of the largest push a context of so many tiles launches (in a batch it is no larger)
+constexpr long long push_warps(int T, int order, long long tiles, int sms) {
+    return tiles * push_split(T, order, tiles, sms) * (push_threads(T) / 32);
+}
+
 }  // namespace hyb

@@ -12,13 +12,14 @@ int main() {
     int T, order, sms;
     long long tiles;
     while (scanf("%%d %%d %%lld %%d", &T, &order, &tiles, &sms) == 4)
-        printf("%%d %%d\\n", hyb::push_split(T, order, tiles, sms), hyb::push_ctas(T, order));
+        printf("%%d %%d %%lld\\n", hyb::push_split(T, order, tiles, sms), hyb::push_ctas(T, order),
+               hyb::push_warps(T, order, tiles, sms));
 }
 """
 
 
 @pytest.fixture(scope="module")
-def rule(tmp_path_factory):
+def table(tmp_path_factory):
     d = tmp_path_factory.mktemp("push_shape")
     (d / "m.cpp").write_text(SRC % ROOT)
     subprocess.run(["g++", "-std=c++17", "-o", str(d / "m"), str(d / "m.cpp")], check=True)
@@ -28,6 +29,16 @@ def rule(tmp_path_factory):
                              capture_output=True, text=True).stdout
         return [tuple(int(v) for v in line.split()) for line in out.splitlines()]
     return run
+
+
+@pytest.fixture(scope="module")
+def rule(table):
+    return lambda rows: [r[:2] for r in table(rows)]
+
+
+@pytest.fixture(scope="module")
+def rule_warps(table):
+    return lambda rows: [r[2] for r in table(rows)]
 
 
 @pytest.mark.parametrize("T", [4, 8])
@@ -50,3 +61,10 @@ def test_quadratic_8_tiles_count_two_ctas_an_sm(rule):
 def test_batches_count_the_tiles_of_all_their_contexts(rule):
     """1, 2, 4 and 8 contexts of 64 tiles side by side: 4, 3, 1 and 1 CTAs a tile."""
     assert [s for s, _ in rule([(8, 1, 64 * n, 152) for n in (1, 2, 4, 8)])] == [4, 3, 1, 1]
+
+
+def test_warps_of_a_launch(rule_warps):
+    """Each warp may leave one chunk of the migration buffer unfinished: the buffer's
+    margin counts the launch's own warps, 4 a CTA on 4^3 tiles and 8 on 8^3 tiles."""
+    rows = [(8, 1, 64, 152), (8, 1, 456, 152), (8, 1, 16384, 152), (4, 1, 64, 152), (4, 1, 4096, 152), (4, 2, 343, 152)]
+    assert rule_warps(rows) == [64 * 4 * 8, 456 * 8, 16384 * 8, 64 * 4 * 4, 4096 * 4, 343 * 2 * 4]
