@@ -716,15 +716,6 @@ __global__ void k_mask_grad(__nv_bfloat16 *__restrict__ d, const __nv_bfloat16 *
     reinterpret_cast<uint4 *>(d)[t] = dv;
 }
 
-// sum the chunk partials in chunk order: out[o] = sum_k part[k][o]
-__global__ void k_sum_parts(const float *__restrict__ part, int nchunks, int nout, float *__restrict__ out) {
-    const int o = blockIdx.x * blockDim.x + threadIdx.x;
-    if (o >= nout) return;
-    float s = 0.0f;
-    for (int k = 0; k < nchunks; ++k) s += part[(long long)k * nout + o];
-    out[o] = s;
-}
-
 __global__ void k_adam(float *__restrict__ w, const float *__restrict__ g, float *__restrict__ m, float *__restrict__ v,
                        int n, float lr, float b1, float b2, float eps, float c1, float c2) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;

@@ -396,8 +396,6 @@ void launch_energy(const GridDev &g, const float *E, const float *B, const SpSet
 
 
 // ---------------------------------------------------------------- network training helpers (classifier.cu)
-// out[o] = sum_k part[k][o], k in increasing order
-__global__ void k_sum_parts(const float *__restrict__ part, int nchunks, int nout, float *__restrict__ out);
 // one Adam step on FP32 masters (c1, c2: the bias corrections 1 - beta^t)
 __global__ void k_adam(float *__restrict__ w, const float *__restrict__ g, float *__restrict__ m, float *__restrict__ v,
                        int n, float lr, float b1, float b2, float eps, float c1, float c2);
@@ -422,10 +420,10 @@ struct DropArgs {
     float scale;
 };
 // a = relu(s + b) [dropout] [+ res]: one thread per cell and 8-channel group;
-// BF16 out (out) or FP32 out (outf); cells = B V
+// BF16 out; cells = B V
 __global__ void k_act_finish(const float *__restrict__ s, const float *__restrict__ bias, int cop, int relu,
                              const __nv_bfloat16 *__restrict__ res, int cres, DropArgs dr, int B, long long V,
-                             __nv_bfloat16 *__restrict__ out, float *__restrict__ outf);
+                             __nv_bfloat16 *__restrict__ out);
 // dz = bf16(G [s + b > 0] keep / (1 - p)): the data gradient at a layer's pre-activation
 __global__ void k_act_dz(const float *__restrict__ G, const float *__restrict__ s, const float *__restrict__ bias,
                          int cop, int relu, DropArgs dr, int B, long long V, __nv_bfloat16 *__restrict__ dz);

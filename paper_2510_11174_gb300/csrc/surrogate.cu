@@ -37,11 +37,10 @@ __device__ __forceinline__ uint32_t keep_bits(uint32_t lin, uint32_t b, uint32_t
     return k;
 }
 
-// a = relu(s + b) [dropout] [+ res]: one thread per cell and 8-channel group;
-// BF16 out (hidden layers) or FP32 out (the last layer, no ReLU)
+// a = relu(s + b) [dropout] [+ res]: one thread per cell and 8-channel group (SwitchNet's layers)
 __global__ void k_act_finish(const float *__restrict__ s, const float *__restrict__ bias, int cop, int relu,
                              const __nv_bfloat16 *__restrict__ res, int cres, DropArgs dr, int B, long long V,
-                             __nv_bfloat16 *__restrict__ out, float *__restrict__ outf) {
+                             __nv_bfloat16 *__restrict__ out) {
     const int ng = cop / 8;
     const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (t >= (long long)B * V * ng) return;
@@ -50,7 +49,7 @@ __global__ void k_act_finish(const float *__restrict__ s, const float *__restric
     const uint32_t keep = dr.thr ? keep_bits((uint32_t)(cell % V), (uint32_t)(cell / V), dr.layer, (uint32_t)grp,
                                              dr.pass, dr.seed, dr.thr)
                                  : 0xFFu;
-    float v[8];
+    __align__(16) __nv_bfloat16 o[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
         const int ch = grp * 8 + j;
@@ -58,18 +57,9 @@ __global__ void k_act_finish(const float *__restrict__ s, const float *__restric
         if (relu) a = fmaxf(a, 0.0f);
         if (dr.thr) a = ((keep >> j) & 1u) ? a * dr.scale : 0.0f;
         if (res && ch < cres) a += __bfloat162float(res[cell * cres + ch]);
-        v[j] = a;
+        o[j] = __float2bfloat16_rn(a);
     }
-    if (outf) {
-        float4 *o4 = reinterpret_cast<float4 *>(outf + cell * cop + grp * 8);
-        o4[0] = make_float4(v[0], v[1], v[2], v[3]);
-        o4[1] = make_float4(v[4], v[5], v[6], v[7]);
-    } else {
-        __align__(16) __nv_bfloat16 o[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) o[j] = __float2bfloat16_rn(v[j]);
-        *reinterpret_cast<uint4 *>(out + cell * cop + grp * 8) = *reinterpret_cast<const uint4 *>(o);
-    }
+    *reinterpret_cast<uint4 *>(out + cell * cop + grp * 8) = *reinterpret_cast<const uint4 *>(o);
 }
 
 // dz = bf16(G [s + b > 0] keep / (1 - p)): the data gradient at layer l's

@@ -331,7 +331,7 @@ hyb_status sn_forward(hyb_switchnet *m, long long n, int pass) {
         if (s != HYB_OK) return s;
         k_act_finish<<<nbs(n * (SN_CO[l] / 8)), RBS, 0, m->stream>>>(
             m->z[l], m->b[l], SN_CO[l], SN_RELU[l], SN_RES[l] ? m->a[l] : nullptr, SN_KP[l], sn_drop(m, l, pass), 1, n,
-            m->a[l + 1], nullptr);
+            m->a[l + 1]);
     }
     k_sn_last<<<nbs(n), RBS, 0, m->stream>>>(m->a[SN_L], m->w[SN_L], m->b[SN_L], n, m->logit);
     cudaError_t e = cudaGetLastError();
