@@ -164,17 +164,17 @@ FIELD_KERNELS = "k_b_half + k_e_yee + k_mur (split Yee step)"
 FLUID_BYTES_PER_NODE = 32
 FLUID_FIELD_BYTES_PER_NODE = 24
 # DRAM read + write per cell of one launch of the 32 -> 32 convolution, from
-# the ncu capture on the 128 x 128 x 64 ramp + slab (67.2 + 19.9 MB for
-# 1,048,576 cells); scaled to a full launch by the cell count
-NCU_CONV_L1_BYTES_PER_CELL = 87.1e6 / 1048576
+# the ncu capture on the 128 x 128 x 64 ramp + slab (60.9 + 10.3 MB for
+# 1,048,576 cells; part of the output stays in L2); scaled to a full launch by the cell count
+NCU_CONV_L1_BYTES_PER_CELL = 71.3e6 / 1048576
 # DRAM read + write per particle of one hybrid-step launch of the push, from
-# the ncu capture on the 128 x 128 x 64 ramp + slab (190.3 + 69.5 MB for its
+# the ncu capture on the 128 x 128 x 64 ramp + slab (151.2 + 63.3 MB for its
 # 4.78 M particles); scaled to a full launch by the particle count
-NCU_PUSH_BYTES_PER_PARTICLE = 259.7e6 / 4784128
+NCU_PUSH_BYTES_PER_PARTICLE = 214.6e6 / 4784128
 # warp instructions of the same capture: the push is bound by instruction
 # issue (its DRAM traffic is the algorithmic bytes), so it is also reported
 # against the SM's issue rate, 4 warp instructions per cycle and SM
-NCU_PUSH_WARP_INST_PER_PARTICLE = 1.074e8 / 4784128
+NCU_PUSH_WARP_INST_PER_PARTICLE = 1.016e8 / 4784128
 N_SM = 152
 
 
@@ -466,7 +466,7 @@ def run_ours(args, rank, world):
         # DRAM bytes and warp instructions of a hybrid-step capture, scaled by
         # the particles (other workloads push ionizing ions and QED leptons: null)
         roofs["push"]["traffic"] = NCU_PUSH_BYTES_PER_PARTICLE * parts
-        roofs["push"]["traffic_note"] = "ncu dram bytes of a 128x128x64 hybrid-step launch scaled by particles"
+        roofs["push"]["traffic_note"] = "ncu dram bytes of a 128x128x64 hybrid-step launch scaled by particles (writes still in L2 at its end are not in them)"
         mhz = clk.get("sm_mhz") or 2070.0
         wi = NCU_PUSH_WARP_INST_PER_PARTICLE * parts
         ach = wi / (phases["push"] * 1e-3)
@@ -479,7 +479,7 @@ def run_ours(args, rank, world):
     if "conv_l1" in roofs:
         # scaled by the nodes the classification evaluated (the launch's tiles cover them and a few more)
         roofs["conv_l1"]["traffic"] = NCU_CONV_L1_BYTES_PER_CELL * (cls.get("classified_cells") or cells)
-        roofs["conv_l1"]["traffic_note"] = "ncu dram bytes of a 128x128x64 launch scaled by the classified cells"
+        roofs["conv_l1"]["traffic_note"] = "ncu dram bytes of a 128x128x64 launch scaled by the classified cells (outputs still in L2 at its end are not in them)"
     # the dominant single kernel (the classification as a whole is reported beside it)
     dom = max((k for k in roofs if k != "classify"), key=lambda k: roofs[k]["share"])
 
