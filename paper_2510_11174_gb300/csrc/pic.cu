@@ -444,10 +444,9 @@ __device__ __forceinline__ void queue_put(float4 *qa, int &n, bool want, const f
 
 // The stochastic events of the push, out of line: a step has few of them, and
 // their code (random numbers, table searches, the writes of new particles) in
-// the particle loop costs every warp instruction cache and registers (spills
-// 188 -> 132 bytes a thread, with the tallies straight to shared memory; a carbon
-// slab of 1.8 M particles with all three events, three runs side by side: five
-// steps 2024 -> 1905 us).
+// the particle loop costs every warp instruction cache and registers (a carbon
+// slab of 1.8 M particles with all three events, three runs side by side, with the
+// tallies straight to shared memory: five steps 2024 -> 1905 us).
 static __device__ __noinline__ void event_spawn(const SpDev *d, float x, float y, float z, float ux, float uy, float uz,
                                                 float w, uint64_t id, int dest, long long step, uint32_t seed, float tau,
                                                 int *status) {
@@ -508,11 +507,13 @@ static __device__ __noinline__ float2 event_pair(const SpDev *sps, int si, const
 // memory before the one rounding to FP32, so the current does not depend on the
 // split.
 // What bounds it, 15.7 M thermal particles (128 x 96 x 80 cells, a third of them
-// crossing a face per step): instruction issue (53 %) and the shared-memory pipe
-// (61 %), 46 B a particle of DRAM traffic.  Measured there, one launch (cold):
-// 1.19 ms with 64-bit atomics and the FP64-pipe conversion, 0.89 ms with the word
-// planes and the one-axis queue, 0.72 ms with the two-conversion digits and the
-// migration chunks; 0.76 M particles of the quadratic shape 0.46 -> 0.25 ms.
+// crossing a face per step): the shared-memory pipe (75 %) and instruction issue
+// (62 %), 56 B a particle of DRAM traffic; at rest 73 and 62 %.  Measured there, one
+// launch (cold): 1.19 ms with 64-bit atomics and the FP64-pipe conversion, 0.89 ms
+// with the word planes and the one-axis queue, 0.72 ms with the two-conversion
+// digits and the migration chunks, 0.68 ms with the prefetched particle in registers
+// (see queue_put; at rest 0.52, 0.62 with the spills, 0.44 ms); 0.76 M particles of
+// the quadratic shape 0.46 -> 0.25 ms.
 template <int T, int ORDER, bool EV, bool SPLIT>
 __global__ void __launch_bounds__(push_threads(T), push_ctas(T, ORDER))
     k_push_deposit(GridDev g, const float *__restrict__ E, const float *__restrict__ B,
